@@ -367,6 +367,20 @@ size_t gram_workspace_bytes(int P, int Q, long long n) {
   return sizeof(double) * (size_t)nchunks * (size_t)(2 * P) * (size_t)(2 * Q);
 }
 
+// Digits on the tensor cores or double-float on the FP32 pipes.  Measured at
+// n = 196608 (double-float -> digits): 72 x 72 pairs 2627 -> 523 us, 24 x 24
+// 736 -> 138, 3 x 24 373 -> 125; at n = 12288: 24 x 24 648 -> 44 us.  Below
+// 8192 rows (32 chunks of 256) there are too few row groups for the SMs and
+// the launches count; a single pair of columns has no tile to fill.
+bool gram_digits_pays(int P, int Q, long long n) { return P * Q > 1 && n >= 8192; }
+
+cudaError_t gram_pairs_fp64(const PairBlock<double>& A, const PairBlock<double>& B, double* G_dev, void* ws,
+                            size_t ws_bytes, cudaStream_t s, bool upper) {
+  if (A.n == B.n && gram_digits_pays(A.cols, B.cols, A.n) && gram_digits_fits(A.cols, B.cols, A.n, ws_bytes))
+    return gram_pairs_digits<double>(A, B, true, G_dev, ws, ws_bytes, s);
+  return gram_pairs<double>(A, B, G_dev, ws, ws_bytes, s, upper);
+}
+
 template <typename R>
 cudaError_t gram_pairs(const PairBlock<R>& A, const PairBlock<R>& B, double* G_dev, void* ws,
                        size_t ws_bytes, cudaStream_t s, bool upper) {

@@ -1,5 +1,6 @@
 // C ABI: plan life cycle, the BdG product, chemical potentials and the
 // deflation bases (Sections 2.3 and 3.1).
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -560,7 +561,9 @@ bdg_status bdg_gram(int dtype, int engine, const void* A, long long lda, int nco
   if (engine == BDG_GRAM_TENSOR && !gram_tc_supported(ncol_a, ncol_b))
     return fail(nullptr, BDG_ERR_UNSUPPORTED, "tensor-core Gram needs 2 ncol_b <= 160");
   cudaStream_t s = (cudaStream_t)stream;
-  const size_t ws_bytes = gram_workspace_bytes(ncol_a, ncol_b, n > 0 ? n : 1);
+  size_t ws_bytes = gram_workspace_bytes(ncol_a, ncol_b, n > 0 ? n : 1);
+  const bool digits = dtype == BDG_C128 && engine == BDG_GRAM_SIMT && gram_digits_pays(ncol_a, ncol_b, n);
+  if (digits) ws_bytes = std::max(ws_bytes, gram_digits_workspace_bytes(ncol_a, ncol_b, n));
   void* ws = nullptr;
   if (cudaMallocAsync(&ws, ws_bytes, s) != cudaSuccess) {
     cudaGetLastError();
@@ -570,7 +573,7 @@ bdg_status bdg_gram(int dtype, int engine, const void* A, long long lda, int nco
   if (dtype == BDG_C128) {
     PairBlock<double> a{(const double2*)A, lda, n, ncol_a}, b{(const double2*)B, ldb, n, ncol_b};
     e = engine == BDG_GRAM_TENSOR ? gram_pairs_tc<double>(a, b, G, ws, ws_bytes, s)
-                                  : gram_pairs<double>(a, b, G, ws, ws_bytes, s, false);
+                                  : gram_pairs_fp64(a, b, G, ws, ws_bytes, s);
   } else {
     PairBlock<float> a{(const float2*)A, lda, n, ncol_a}, b{(const float2*)B, ldb, n, ncol_b};
     e = engine == BDG_GRAM_TENSOR ? gram_pairs_tc<float>(a, b, G, ws, ws_bytes, s)

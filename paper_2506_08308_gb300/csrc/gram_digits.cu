@@ -1,0 +1,451 @@
+// Tall-skinny Gram G = A^T B of two pair blocks on the tensor cores
+// (tcgen05.mma kind::f16, accumulators in tensor memory), from exact digits
+// (digits.cuh): FP64 accuracy with six digits per element (26 digit
+// products), FP32 accuracy with four (10 products).
+//
+// A CTA owns a tile of 128 x NT real columns and a range of row chunks of
+// CHUNK = 256 rows.  Every column has one exponent per chunk (k_col_exp),
+// against which its values are cut into digits; within a chunk the products
+// of each digit weight add up in one FP32 accumulator, exactly for the four
+// leading weights (256 rows x 4 pairs x 2^14 = 2^24), to 2^-24 of a part
+// below 2^-32 of the result for the others.  After a chunk the
+// accumulators are read back and added, error-free down to the second float,
+// to a double-float sum per output in registers; the CTA writes its sum as
+// FP64, and the CTAs' partial sums are added in FP64 in a fixed order.
+//
+// Why: a double-float multiply-add is 15 FP32 instructions, so the same
+// contraction in double-float is bound by the FP32 pipe at 5 TFLOP/s (and
+// measured at 3).  Here the arithmetic is 26 (10) FP16 products per
+// multiply-add on the tensor cores, and cutting the digits about 30 integer
+// instructions per element and tile.  72 x 72 pairs of 196608 rows: 2627 ->
+// 520 us (15.7 TFLOP/s of FP64 work), error 5e-15 -> 2e-15 of |G|; 24 x 24:
+// 736 -> 138 us.  What bounds it now is the integer pipe of the producer
+// warps (52 % of its rate, 3300 clocks per 32-row stage against 2300 of the
+// MMAs, each of which reads 5.5 KB of operands at 128 bytes per clock); the
+// pass over the exponents takes 72 us at 80 % of the DRAM rate.
+//
+// Operand tiles are MN-major without swizzle: a core matrix holds 8 rows (K)
+// of 8 neighbouring real columns (16 bytes), so that a thread that has one
+// row of four complex columns stores 16 bytes per digit, a warp reads 32
+// consecutive rows of a column and its stores cover whole bank cycles.
+#include <algorithm>
+
+#include "blas.cuh"
+#include "digits.cuh"
+
+namespace bdg {
+
+namespace {
+
+constexpr int TM = 128;      // A real columns per CTA (MMA M)
+constexpr int TBK = 32;      // rows per pipeline stage (two MMA K steps of 16)
+constexpr int TSTAGES = 3;   // stages in flight
+constexpr int PWARPS = 16;   // warps that cut digits and read back; one more issues the MMAs
+constexpr int TTHREADS = 32 * (PWARPS + 1);
+constexpr int CHUNK = 256;   // rows per exponent and per read-back
+constexpr int STEPS = CHUNK / TBK;
+// digit weights kept: with six digits the seventh as well, whose five pairs
+// would otherwise be the largest error
+template <int ND> constexpr int weights() { return ND == 6 ? 7 : ND; }
+inline int padded8(int cols) { return (cols + 7) / 8 * 8; }
+
+// exps[chunk * ld + 2 c + part]: largest biased exponent of the column's real
+// (imaginary) parts in the chunk; one warp per chunk and complex column, the
+// columns up to ld (2 cols rounded up to 8) are zero
+template <typename R>
+__global__ void __launch_bounds__(256) k_col_exp(PairBlock<R> X, int nchunks, int ld, short* __restrict__ exps) {
+  typedef typename CT<R>::T T;
+  const int warp = (int)((blockIdx.x * 256LL + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  const int c = warp / nchunks, chunk = warp - c * nchunks;
+  if (2 * c >= ld) return;
+  if (c >= X.cols) {
+    if (lane == 0) *reinterpret_cast<short2*>(exps + (long long)chunk * ld + 2 * c) = make_short2(0, 0);
+    return;
+  }
+  const T* p = X.p + (long long)c * X.ld + (long long)chunk * CHUNK;
+  const int rows = (int)min((long long)CHUNK, X.n - (long long)chunk * CHUNK);
+  int ex = 0, ey = 0;
+#pragma unroll
+  for (int k = 0; k < CHUNK / 32; ++k) {
+    const int r = lane + 32 * k;
+    if (r < rows) {
+      const T v = p[r];
+      ex = max(ex, exponent_of(v.x));
+      ey = max(ey, exponent_of(v.y));
+    }
+  }
+  ex = __reduce_max_sync(0xffffffffu, ex);
+  ey = __reduce_max_sync(0xffffffffu, ey);
+  if (lane == 0) *reinterpret_cast<short2*>(exps + (long long)chunk * ld + 2 * c) = make_short2((short)ex, (short)ey);
+}
+
+// 2^e as a float for e <= 0, 0 below the normal range
+__device__ __forceinline__ float pow2_neg(int e) { return e < -126 ? 0.f : __int_as_float((e + 127) << 23); }
+
+// Work of one producer warp in every stage: four complex columns, 32 rows.
+// Columns past the block's last are read from the last one: their digits land
+// in rows (columns) of the tile that nothing reads.
+template <typename R>
+struct RowTask {
+  const typename CT<R>::T* p;  // first column, the lane's row of the next load
+  long long ld;                // column stride, 0 past the last column
+  int c1, c2, c3;              // columns 1..3 in units of ld
+  const short* e;              // exponents of the chunk of the next load
+  typename CT<R>::T v[4];
+  uint4 ev;                    // eight exponents (shorts)
+  __device__ __forceinline__ void start(const PairBlock<R>& X, const short* exps, int c0, long long r) {
+    const int last = X.cols - 1 - c0;
+    p = X.p + (long long)c0 * X.ld + r;
+    ld = X.ld;
+    c1 = min(1, last);
+    c2 = min(2, last);
+    c3 = min(3, last);
+    e = exps + 2 * c0;
+  }
+  __device__ __forceinline__ void load(bool in) {
+    ev = *reinterpret_cast<const uint4*>(e);
+    if (in) {
+      v[0] = p[0];
+      v[1] = p[c1 * ld];
+      v[2] = p[c2 * ld];
+      v[3] = p[c3 * ld];
+    } else {
+      v[0] = v[1] = v[2] = v[3] = mk((R)0, (R)0);
+    }
+    p += TBK;
+  }
+};
+// digits of eight real columns at one row: 16 bytes per digit tile
+template <typename R, int ND>
+__device__ __forceinline__ void store_task(const RowTask<R>& x, uint8_t* base, uint32_t tile_bytes) {
+  const unsigned e[4] = {x.ev.x, x.ev.y, x.ev.z, x.ev.w};
+  uint32_t d[4][ND];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    digit_pairs<ND>(to_fixed<ND>(x.v[q].x, (int)(e[q] << 20)), to_fixed<ND>(x.v[q].y, (int)(e[q] << 4)), d[q]);
+#pragma unroll
+  for (int k = 0; k < ND; ++k)
+    *reinterpret_cast<uint4*>(base + k * tile_bytes) = make_uint4(d[0][k], d[1][k], d[2][k], d[3][k]);
+}
+
+__device__ __forceinline__ void bar_init(uint64_t* bar, int count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// part[group][i][j] for a tile of mw <= 128 x nw <= NT real columns over the chunks of blockIdx.z.  Sixteen producer warps cut the digits of
+// the next stage while one thread issues the MMAs of the last; the read-back
+// of a chunk comes after the next chunk's first stage is in place.  A wait
+// that runs out writes NaN.
+template <typename R, int ND, int NT>
+__global__ void __launch_bounds__(TTHREADS, 1)
+    k_gram_digits(PairBlock<R> A, PairBlock<R> B, const short* __restrict__ expA, const short* __restrict__ expB, int ldea,
+              int ldeb, int mw, int nw, int nchunks, int chunks_per_group, double* __restrict__ part) {
+  constexpr int NW = weights<ND>();
+  constexpr uint32_t A_TILE = TM * TBK * 2, B_TILE = NT * TBK * 2, STAGE = ND * (A_TILE + B_TILE);
+  constexpr uint32_t NCOLS = NW * NT <= 32 ? 32 : NW * NT <= 64 ? 64 : NW * NT <= 128 ? 128 : NW * NT <= 256 ? 256 : 512;
+  static_assert(NW * NT <= 512 && NT % 16 == 0, "one accumulator per digit weight");
+  constexpr int NQ = NT / 4;  // output columns per thread
+  extern __shared__ __align__(1024) uint8_t smem[];
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + TSTAGES * STAGE);
+  uint64_t* empty = full + TSTAGES;
+  uint64_t* acc_full = empty + TSTAGES;
+  uint64_t* acc_free = acc_full + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_free + 1);
+  int* ra = reinterpret_cast<int*>(tmem_slot + 2);  // [TM] largest exponents of the group's chunks
+  int* rb = ra + TM;                                // [NT]
+  // (the shuffle tells the compiler that the warp index is uniform)
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const int i0 = blockIdx.x * mw, j0 = blockIdx.y * nw;
+  const int Q2 = 2 * B.cols, i1 = min(2 * A.cols, i0 + mw), j1 = min(Q2, j0 + nw);
+  const int ch0 = blockIdx.z * chunks_per_group, ch1 = min(nchunks, ch0 + chunks_per_group);
+
+  if (warp == PWARPS) tmem_alloc(tmem_slot, NCOLS);
+  if (tid == 0) {
+    for (int s = 0; s < TSTAGES; ++s) {
+      bar_init(&full[s], PWARPS);
+      bar_init(&empty[s], 1);
+    }
+    bar_init(acc_full, 1);
+    bar_init(acc_free, PWARPS);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  for (int c = tid; c < TM + NT; c += TTHREADS) {
+    const bool isA = c < TM;
+    const int col = isA ? i0 + c : j0 + c - TM, ld = isA ? ldea : ldeb;
+    const short* e = isA ? expA : expB;
+    int m = 0;
+    if (col < (isA ? i1 : j1))
+      for (int ch = ch0; ch < ch1; ++ch) m = max(m, (int)e[(long long)ch * ld + col]);
+    (isA ? ra : rb)[isA ? c : c - TM] = m;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const int nsteps = max(0, ch1 - ch0) * STEPS;
+  bool lost = false;
+
+  if (warp == PWARPS) {
+    const uint32_t idesc = mma_idesc_f16(TM, NT, true, true);
+    const bool leader = elect_one();
+    for (int step = 0; step < nsteps; ++step) {
+      const int st = step % TSTAGES, u = step / TSTAGES;
+      if (!mma_wait(&full[st], (uint32_t)(u & 1))) lost = true;
+      // accumulators of the chunk before have been read back
+      if (step % STEPS == 0 && step > 0 && !mma_wait(acc_free, (uint32_t)((step / STEPS - 1) & 1))) lost = true;
+      tc_fence_after();
+      if (leader) {
+        const uint32_t sa = smem_u32(smem + st * STAGE), sb = sa + ND * A_TILE;
+        const uint64_t da = mma_desc(sa, (TM / 8) * 128, 128), db = mma_desc(sb, (NT / 8) * 128, 128);
+        const bool first = step % STEPS == 0;
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+          for (int i = 0; i < ND; ++i)
+#pragma unroll
+            for (int j = 0; j < ND && i + j < NW; ++j)
+              mma_f16(tmem + (uint32_t)((i + j) * NT), da + ((i * A_TILE + kk * 2 * (TM / 8) * 128) >> 4),
+                      db + ((j * B_TILE + kk * 2 * (NT / 8) * 128) >> 4), idesc,
+                      !(first && kk == 0 && (i == 0 || (j == ND - 1 && i + j >= ND && i == NW - ND))));
+        mma_commit(&empty[st]);
+        if (step % STEPS == STEPS - 1) mma_commit(acc_full);
+      }
+      __syncwarp();
+    }
+  } else {
+    // tasks of a stage: groups of four complex columns of A, then of B, one or
+    // two to a warp.  The loads of a task are issued a stage ahead.
+    const int na = (i1 - i0 + 7) / 8, nt = na + (j1 - j0 + 7) / 8;
+    RowTask<R> x[2];
+    const long long r_first = (long long)ch0 * CHUNK + lane;
+    auto start = [&](int q) {
+      const int t = warp + PWARPS * q;
+      if (t < na) x[q].start(A, expA + (long long)ch0 * ldea, i0 / 2 + 4 * t, r_first);
+      else if (t < nt) x[q].start(B, expB + (long long)ch0 * ldeb, j0 / 2 + 4 * (t - na), r_first);
+    };
+    auto fetch = [&](int step, int q) {
+      const int t = warp + PWARPS * q;
+      if (t >= nt || step >= nsteps) return;
+      if (step % STEPS == 0 && step > 0) x[q].e += t < na ? ldea : ldeb;
+      x[q].load(r_first + (long long)step * TBK < A.n);
+    };
+    float hi[NQ], lo[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) hi[q] = lo[q] = 0.f;
+    const int quarter = warp & 3, jq = (warp >> 2) * NQ;
+    const int row = 32 * quarter + lane;
+    const uint32_t tlane = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)jq;
+    auto read_back = [&](int chunk) {  // chunk of this group
+      if (!mma_wait(acc_full, (uint32_t)(chunk & 1))) lost = true;
+      tc_fence_after();
+      const int ch = ch0 + chunk;
+      // (a column without a normal number in the chunk counts as zero)
+      const int xa = i0 + row < i1 ? (int)expA[(long long)ch * ldea + i0 + row] : 0;
+      const float fa = xa ? pow2_neg(xa - ra[row]) : 0.f;
+#pragma unroll
+      for (int c0 = 0; c0 < NQ; c0 += 4) {
+        float v[NW][4];
+#pragma unroll
+        for (int w = 0; w < NW; ++w) tmem_ld4(tlane + (uint32_t)(w * NT + c0), v[w]);
+        int e[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int xb = j0 + jq + c0 + q < j1 ? (int)expB[(long long)ch * ldeb + j0 + jq + c0 + q] : 0;
+          e[q] = xb ? xb - rb[jq + c0 + q] : -4096;
+        }
+        tmem_ld_wait();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float g = fa * pow2_neg(e[q]);
+          // three leading weights by error-free sums, the rest in one float
+          float s = hi[c0 + q], err = 0.f;
+#pragma unroll
+          for (int w = 0; w < 3; ++w) {
+            const float t = v[w][q] * (g * (w == 0 ? 1.f : w == 1 ? 0x1p-8f : 0x1p-16f));
+            const float n = __fadd_rn(s, t), b = __fsub_rn(n, s);
+            err = __fadd_rn(err, __fadd_rn(__fsub_rn(s, __fsub_rn(n, b)), __fsub_rn(t, b)));
+            s = n;
+          }
+          float tail = v[NW - 1][q];
+#pragma unroll
+          for (int w = NW - 2; w >= 3; --w) tail = fmaf(tail, 0x1p-8f, v[w][q]);
+          const float l = __fadd_rn(lo[c0 + q], fmaf(tail, g * 0x1p-24f, err));
+          const float n = __fadd_rn(s, l);
+          lo[c0 + q] = __fsub_rn(l, __fsub_rn(n, s));
+          hi[c0 + q] = n;
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) bar_arrive(acc_free);
+    };
+    auto produce = [&](int step, int q) {
+      const int st = step % TSTAGES, t = warp + PWARPS * q;
+      if (t >= nt) return;
+      // core matrix (row group lane / 8, column group g) at ((lane / 8) groups + g) 128, 16 bytes per row
+      uint8_t* base = t < na ? smem + st * STAGE + ((lane >> 3) * (TM / 8) + t) * 128
+                             : smem + st * STAGE + ND * A_TILE + ((lane >> 3) * (NT / 8) + t - na) * 128;
+      store_task<R, ND>(x[q], base + (lane & 7) * 16, t < na ? A_TILE : B_TILE);
+    };
+    start(0);
+    start(1);
+    fetch(0, 0);
+    fetch(0, 1);
+    for (int step = 0; step < nsteps; ++step) {
+      const int st = step % TSTAGES;
+      // the MMAs that read this stage (committed TSTAGES steps ago) are done
+      if (step >= TSTAGES && !mma_wait(&empty[st], (uint32_t)((step / TSTAGES - 1) & 1))) lost = true;
+      if (step > STEPS && step % STEPS == TSTAGES - 1) read_back(step / STEPS - 1);
+      produce(step, 0);
+      fetch(step + 1, 0);
+      produce(step, 1);
+      fetch(step + 1, 1);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) bar_arrive(&full[st]);
+    }
+    if (nsteps > 0) read_back(nsteps / STEPS - 1);
+    const int i = i0 + row;
+    if (i < i1) {
+      const int er = ra[row];
+      double* out = part + ((long long)blockIdx.z * 2 * A.cols + i) * Q2;
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        const int j = j0 + jq + q;
+        if (j >= j1) continue;
+        const int e2 = rb[jq + q];
+        const bool bad = lost || er >= 2047 || e2 >= 2047;  // infinities and NaN
+        out[j] = bad ? (double)NAN : scalbn((double)hi[q] + (double)lo[q], product_unit<ND>(er, e2));
+      }
+    }
+  }
+  const bool any_lost = __syncthreads_or(lost) != 0;
+  if (any_lost && warp != PWARPS && i0 + 32 * (warp & 3) + lane < i1) {  // a wait of another warp ran out
+    double* out = part + ((long long)blockIdx.z * 2 * A.cols + i0 + 32 * (warp & 3) + lane) * Q2;
+    for (int j = j0 + (warp >> 2) * NQ; j < min(j1, j0 + ((warp >> 2) + 1) * NQ); ++j) out[j] = (double)NAN;
+    mma_wait(acc_full, (uint32_t)((nsteps / STEPS - 1) & 1));  // the MMAs may still run: wait, bounded
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == PWARPS) tmem_free(tmem, NCOLS);
+}
+
+// G[e] = sum over groups, in a fixed order: thread (x, y) of a 32 x 8 block
+// sums groups y, y + 8, ... of output e (independent loads in flight), then
+// the eight sums are added in order of y.
+__global__ void __launch_bounds__(256) k_gram_digits_reduce(const double* __restrict__ part, int ngroups, int nout,
+                                                        double* __restrict__ G) {
+  __shared__ double t[8][33];
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  const int e = blockIdx.x * 32 + x;
+  double s = 0.0;
+  if (e < nout)
+#pragma unroll 4
+    for (int c = y; c < ngroups; c += 8) s += part[(long long)c * nout + e];
+  t[y][x] = s;
+  __syncthreads();
+  if (y == 0 && e < nout) {
+    double g = t[0][x];
+#pragma unroll
+    for (int q = 1; q < 8; ++q) g += t[q][x];
+    G[e] = g;
+  }
+}
+
+struct Shape {
+  int mt, nt, mw, nw, NT, nchunks, groups, cpg;
+  size_t part_bytes, exp_bytes;
+};
+
+// column tiles, row groups (one CTA per SM, fewer if the workspace holds
+// fewer partial sums) and workspace of a Gram
+template <int ND>
+Shape shape_of(int P, int Q, long long n, size_t ws_bytes = SIZE_MAX) {
+  Shape s;
+  const int P2 = 2 * P, Q2 = 2 * Q, cap = ND == 6 ? 64 : 128;
+  s.mt = (P2 + TM - 1) / TM;
+  s.nt = (Q2 + cap - 1) / cap;
+  // tiles of equal width (the MMA takes 128 x NT columns whatever the tile holds)
+  s.mw = padded8((P2 + s.mt - 1) / s.mt);
+  s.nw = padded8((Q2 + s.nt - 1) / s.nt);
+  s.NT = s.nw <= 16 ? 16 : s.nw <= 48 ? 48 : ND == 6 ? 64 : s.nw <= 80 ? 80 : 128;
+  s.nchunks = (int)((n + CHUNK - 1) / CHUNK);
+  s.exp_bytes = sizeof(short) * (size_t)s.nchunks * (padded8(P2) + padded8(Q2));
+  const size_t per = sizeof(double) * (size_t)P2 * Q2;
+  const size_t fit = ws_bytes > s.exp_bytes + 16 ? (ws_bytes - s.exp_bytes - 16) / per : 0;
+  const int want = (int)std::max<size_t>(1, std::min<size_t>(152 / (s.mt * s.nt), fit));
+  s.cpg = (s.nchunks + want - 1) / want;
+  s.groups = (s.nchunks + s.cpg - 1) / s.cpg;
+  s.part_bytes = (sizeof(double) * (size_t)s.groups * P2 * Q2 + 15) / 16 * 16;
+  return s;
+}
+
+template <typename R, int ND, int NT>
+cudaError_t launch(const PairBlock<R>& A, const PairBlock<R>& B, const Shape& h, void* ws, cudaStream_t s) {
+  const size_t smem = (size_t)TSTAGES * ND * (TM + NT) * TBK * 2 + 8 * (2 * TSTAGES + 2) + 8 + sizeof(int) * (TM + NT);
+  cudaError_t e = allow_dynamic_smem((const void*)k_gram_digits<R, ND, NT>, smem);
+  if (e != cudaSuccess) return e;
+  const int lda = padded8(2 * A.cols), ldb = padded8(2 * B.cols);
+  short* ea = (short*)((char*)ws + h.part_bytes);
+  k_gram_digits<R, ND, NT><<<dim3(h.mt, h.nt, h.groups), TTHREADS, smem, s>>>(
+      A, B, ea, ea + (size_t)h.nchunks * lda, lda, ldb, h.mw, h.nw, h.nchunks, h.cpg, (double*)ws);
+  return cudaGetLastError();
+}
+
+template <typename R, int ND>
+cudaError_t gram_digits(const PairBlock<R>& A, const PairBlock<R>& B, double* G_dev, void* ws, size_t ws_bytes,
+                        cudaStream_t s) {
+  if (A.n != B.n) return cudaErrorInvalidValue;
+  const int P2 = 2 * A.cols, Q2 = 2 * B.cols;
+  if (P2 == 0 || Q2 == 0) return cudaSuccess;
+  if (A.n == 0) return cudaMemsetAsync(G_dev, 0, sizeof(double) * P2 * Q2, s);
+  const Shape h = shape_of<ND>(A.cols, B.cols, A.n, ws_bytes);
+  if (ws_bytes < h.part_bytes + h.exp_bytes) return cudaErrorInvalidValue;
+  short* ea = (short*)((char*)ws + h.part_bytes);
+  const int lda = padded8(P2), ldb = padded8(Q2);
+  k_col_exp<R><<<(unsigned)(((long long)h.nchunks * (lda / 2) + 7) / 8), 256, 0, s>>>(A, h.nchunks, lda, ea);
+  k_col_exp<R><<<(unsigned)(((long long)h.nchunks * (ldb / 2) + 7) / 8), 256, 0, s>>>(B, h.nchunks, ldb,
+                                                                                       ea + (size_t)h.nchunks * lda);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  if (h.NT == 16) e = launch<R, ND, 16>(A, B, h, ws, s);
+  else if (h.NT == 48) e = launch<R, ND, 48>(A, B, h, ws, s);
+  else if constexpr (ND == 6) e = launch<R, ND, 64>(A, B, h, ws, s);
+  else if (h.NT == 80) e = launch<R, ND, 80>(A, B, h, ws, s);
+  else e = launch<R, ND, 128>(A, B, h, ws, s);
+  if (e != cudaSuccess) return e;
+  const int nout = P2 * Q2;
+  k_gram_digits_reduce<<<(nout + 31) / 32, 256, 0, s>>>((const double*)ws, h.groups, nout, G_dev);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t gram_digits_workspace_bytes(int P, int Q, long long n) {
+  if (P <= 0 || Q <= 0 || n <= 0) return 0;
+  const Shape a = shape_of<4>(P, Q, n), b = shape_of<6>(P, Q, n);
+  return 16 + std::max(a.part_bytes + a.exp_bytes, b.part_bytes + b.exp_bytes);
+}
+
+bool gram_digits_fits(int P, int Q, long long n, size_t ws_bytes) {
+  const Shape a = shape_of<4>(P, Q, n, ws_bytes), b = shape_of<6>(P, Q, n, ws_bytes);
+  return std::max(a.part_bytes + a.exp_bytes, b.part_bytes + b.exp_bytes) <= ws_bytes;
+}
+
+template <typename R>
+cudaError_t gram_pairs_digits(const PairBlock<R>& A, const PairBlock<R>& B, bool fp64, double* G_dev, void* ws,
+                              size_t ws_bytes, cudaStream_t s) {
+  if constexpr (sizeof(R) == 8)
+    if (fp64) return gram_digits<R, 6>(A, B, G_dev, ws, ws_bytes, s);
+  return gram_digits<R, 4>(A, B, G_dev, ws, ws_bytes, s);
+}
+
+template cudaError_t gram_pairs_digits<float>(const PairBlock<float>&, const PairBlock<float>&, bool, double*, void*,
+                                              size_t, cudaStream_t);
+template cudaError_t gram_pairs_digits<double>(const PairBlock<double>&, const PairBlock<double>&, bool, double*,
+                                               void*, size_t, cudaStream_t);
+
+}  // namespace bdg

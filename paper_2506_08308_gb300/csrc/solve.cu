@@ -335,16 +335,23 @@ class Solver {
   // ---- primitive wrappers ----------------------------------------------
   // G (2P x 2Q) of real columns, FP64 on device
   // Grams for which FP32 accuracy suffices -- every Gram of the FP32 phase,
-  // and the first pass of the two-pass Gram-Schmidt, whose second pass
-  // (double-float) removes what the first leaves -- run on the tensor cores
-  // (split-BF16 slices, FP32 accumulation); the rest in double-float.
+  // and the first pass of the two-pass Gram-Schmidt, whose second pass (FP64)
+  // removes what the first leaves -- take four digits per element on the
+  // tensor cores, the others six where gram_digits_pays says so (else
+  // double-float; BDG_GRAM_TC=0: double-float and FP32 SIMT throughout).
   bool tc_ = !getenv("BDG_GRAM_TC") || atoi(getenv("BDG_GRAM_TC")) != 0;
   static constexpr long long TC_MIN_ROWS = 2048;
   bdg_status gram(const PairBlock<R>& A, const PairBlock<R>& B, double* G, bool upper = false,
                   bool fp32_enough = sizeof(R) == 4) {
-    if (tc_ && fp32_enough && A.n >= TC_MIN_ROWS && gram_tc_supported(A.cols, B.cols)) {
-      BDG_CUDA_TRY(plan_, gram_pairs_tc<R>(A, B, G, gws_, gws_bytes_, s_));
+    if (tc_ && fp32_enough && A.n >= TC_MIN_ROWS && gram_digits_fits(A.cols, B.cols, A.n, gws_bytes_)) {
+      BDG_CUDA_TRY(plan_, gram_pairs_digits<R>(A, B, false, G, gws_, gws_bytes_, s_));
       return BDG_OK;
+    }
+    if constexpr (sizeof(R) == 8) {
+      if (tc_) {
+        BDG_CUDA_TRY(plan_, gram_pairs_fp64(A, B, G, gws_, gws_bytes_, s_, upper));
+        return BDG_OK;
+      }
     }
     BDG_CUDA_TRY(plan_, gram_pairs<R>(A, B, G, gws_, gws_bytes_, s_, upper));
     return BDG_OK;
