@@ -226,12 +226,6 @@ __global__ void __launch_bounds__(W / 2 * Split<N>::N1, N <= 256 ? 512 / (W / 2 
   }
 }
 
-static int log2i(long long v) {  // v a power of two
-  int b = 0;
-  while ((1LL << b) < v) ++b;
-  return b;
-}
-
 template <int N>
 static cudaError_t launch_row2(const ApplyArgs<float>& g, cudaStream_t s) {
   constexpr int RP = 32 / Split<N>::N1;

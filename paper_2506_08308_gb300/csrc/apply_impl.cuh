@@ -272,6 +272,12 @@ __global__ void __launch_bounds__(W * Split<N>::N1, (sizeof(R) == 4 && N <= 256)
 // ---------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------
+static int log2i(long long v) {  // v a power of two
+  int b = 0;
+  while ((1LL << b) < v) ++b;
+  return b;
+}
+
 template <int N, typename R>
 static cudaError_t launch_row(const ApplyArgs<R>& g, cudaStream_t s) {
   typedef typename CT<R>::T T;
@@ -332,27 +338,5 @@ static cudaError_t launch_axis(const ApplyArgs<R>& g, int ax, cudaStream_t s) {
     case 1024: return FN<1024, R>(__VA_ARGS__);               \
     default: return cudaErrorInvalidValue;                    \
   }
-
-template <typename R>
-static cudaError_t row_dispatch(const ApplyArgs<R>& g, cudaStream_t s) {
-  BDG_DISPATCH_N(g.grid->n[g.grid->dim - 1], launch_row, g, s)
-}
-template <typename R>
-static cudaError_t axis_dispatch(const ApplyArgs<R>& g, int ax, cudaStream_t s) {
-  BDG_DISPATCH_N(g.grid->n[ax], launch_axis, g, ax, s)
-}
-
-template <typename R>
-cudaError_t apply_launch(const ApplyArgs<R>& g, cudaStream_t s) {
-  if (g.nvec <= 0) return cudaSuccess;
-  cudaError_t e = row_dispatch<R>(g, s);
-  if (e != cudaSuccess) return e;
-  for (int ax = g.grid->dim - 2; ax >= 0; --ax) {
-    e = axis_dispatch<R>(g, ax, s);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
 
 }  // namespace bdg

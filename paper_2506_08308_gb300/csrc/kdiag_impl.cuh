@@ -11,6 +11,7 @@
 
 #include "common.cuh"
 #include "fft.cuh"
+#include "fft_spread.cuh"
 #include "kdiag.cuh"
 
 namespace bdg {
@@ -165,10 +166,88 @@ __global__ void __launch_bounds__(W * Split<N>::N1) k_kd_strided(const typename 
   for (int n2 = 0; n2 < N2; ++n2) yl[(long long)(j + N1 * n2) * st] = a[n2];
 }
 
+// Both kinds of passes for few lines (fft_spread.cuh): contiguous lines have
+// st = 1; the others are walked with neighbouring lines in neighbouring
+// threads.  x may equal y.
+template <int N, typename R>
+__global__ void __launch_bounds__(Spread<N, typename CT<R>::T>::FT)
+    k_kd_spread(const typename CT<R>::T* x, typename CT<R>::T* y, long long nlines, long long npts, long long st,
+                int line_bits, int st_bits, const typename CT<R>::T* __restrict__ twg, int mode, KdCoef c, int axis) {
+  typedef typename CT<R>::T T;
+  typedef Spread<N, T> L;
+  constexpr int TH = L::TH, WL = L::WARP_LINES, FT = L::FT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* ex = reinterpret_cast<T*>(smem_raw);  // [WL][2 N]
+  const int l = st == 1 ? threadIdx.x / TH : threadIdx.x % WL, t = st == 1 ? threadIdx.x % TH : threadIdx.x / WL;
+  const long long line = (long long)blockIdx.x * WL + l;
+  const bool act = line < nlines;
+  const long long ln = act ? line : 0;
+  const long long in = ln & ((1LL << line_bits) - 1), inner = in & (st - 1);
+  const long long base = (ln >> line_bits) * npts + (in >> st_bits) * (N * st) + inner + t * st;
+  T a[4];
+  L f;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) a[k] = x[base + TH * k * st];
+  f.load_twiddles(t, twg);
+  T* e = ex + l * 2 * N;
+  auto go = [&](auto sync) {
+    if (mode != KD_INV) f.template run<-1>(a, t, e, sync);
+    if (mode == KD_FMI) {
+      double extra = 0.0;  // |mu|^2 of the other axes (axis 0: their spectral indices are the place in the plane)
+      if (axis == 0 && c.n[1] > 1) {
+        const int n2 = c.n[2] > 1 ? c.n[2] : 1;
+        const int i2 = (int)(inner % n2), i1 = (int)(inner / n2);
+        const int k1 = i1 < c.n[1] / 2 ? i1 : i1 - c.n[1], k2 = i2 < n2 / 2 ? i2 : i2 - n2;
+        extra = c.kappa[1] * (double)(k1 * k1) + (n2 > 1 ? c.kappa[2] * (double)(k2 * k2) : 0.0);
+      }
+      const R base_d = (R)(c.shift + c.scale * extra), sk = (R)(c.scale * (axis == 0 ? c.kappa[0] : axis == 1 ? c.kappa[1] : c.kappa[2]));
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int kk = kidx<N>(t + TH * k);
+        a[k] = a[k] * ((R)c.norm / (base_d + sk * (R)(kk * kk)));
+      }
+    }
+    if (mode != KD_FWD) f.template run<1>(a, t, e, sync);
+  };
+  if constexpr (FT == 32) go(SpreadWarp());
+  else go(SpreadBar<FT>());
+  if (act) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) y[base + TH * k * st] = a[k];
+  }
+}
+
+inline int kd_log2(long long v) {  // v a power of two
+  int b = 0;
+  while ((1LL << b) < v) ++b;
+  return b;
+}
+
+template <int N, typename R>
+static cudaError_t kd_spread(const KdArgs<R>& g, const KdCoef& c, int ax, long long st, const typename CT<R>::T* x,
+                             typename CT<R>::T* y, int mode) {
+  typedef Spread<N, typename CT<R>::T> L;
+  const size_t sm = sizeof(typename CT<R>::T) * (size_t)L::WARP_LINES * 2 * N;
+  cudaError_t e = allow_dynamic_smem((const void*)k_kd_spread<N, R>, sm);
+  if (e != cudaSuccess) return e;
+  const long long per = g.grid->npts / N, nlines = per * g.nplanes;
+  k_kd_spread<N, R><<<(unsigned)((nlines + L::WARP_LINES - 1) / L::WARP_LINES), L::FT, sm, g.stream>>>(
+      x, y, nlines, g.grid->npts, st, kd_log2(per), kd_log2(st), g.tw[ax], mode, c, ax);
+  return cudaGetLastError();
+}
+
+// FP64 passes over few lines go four points per thread (as the product's do)
+template <typename R>
+static bool kd_few_lines(const KdArgs<R>& g, int n) {
+  return sizeof(R) == 8 && g.grid->npts / n * g.nplanes <= FEW_LINES;
+}
+
 template <int N, typename R>
 static cudaError_t kd_contig(const KdArgs<R>& g, const KdCoef& c, const typename CT<R>::T* x,
                              typename CT<R>::T* y, int mode) {
   typedef typename CT<R>::T T;
+  if constexpr (sizeof(R) == 8)
+    if (kd_few_lines(g, N)) return kd_spread<N, R>(g, c, g.grid->dim - 1, 1, x, y, mode);
   constexpr int N1 = Split<N>::N1, LPC = 8 * (32 / N1);
   const size_t sm = sizeof(T) * ((size_t)N + (size_t)LPC * N);
   auto kern = k_kd_contig<N, R>;
@@ -201,6 +280,8 @@ static cudaError_t kd_strided(const KdArgs<R>& g, const KdCoef& c, int ax, const
   typedef typename CT<R>::T T;
   long long st = 1;
   for (int a = ax + 1; a < g.grid->dim; ++a) st *= g.grid->n[a];
+  if constexpr (sizeof(R) == 8)
+    if (kd_few_lines(g, N)) return kd_spread<N, R>(g, c, ax, st, x, y, mode);
   const size_t per_line = sizeof(T) * (N + 1);
   long long w = per_line * 16 <= 80 * 1024 ? 16 : per_line * 8 <= 80 * 1024 ? 8 : 4;
   if (w > st) w = st;

@@ -41,3 +41,34 @@ def test_apply_f32_lines(n):
             assert err < 30 * 2.0 ** -24, (mode, nvec, err)
             assert buf[0] == 0 and buf[-1] == 0
     plan.close()
+
+
+@pytest.mark.parametrize("n", GRIDS, ids=lambda n: "x".join(map(str, n)))
+def test_apply_f64_few_lines(n):
+    """FP64 products of one and three vectors (few lines: four points per
+    thread) against the oracle, and those of a block of more than 5000 lines
+    (the other kernels) against its vectors taken one by one."""
+    torch = need_torch_cuda()
+    from oracle import apply as ap
+    from paper_2506_08308_gb300 import bdg
+    d = len(n)
+    w = synth.Workload("lines", n, (-4.0,) * d, (4.0,) * d, (1.0, 1.3, 0.8)[:d], 20.0, -1.0, 0.05, 0.1, gs_seed=3)
+    V, phi, mu = synth.potential(w), synth.initial_spinor(w) * 0.3, np.array([1.1, 0.9, 1.3])
+    op = ap.Operator(w, phi, V, mu)
+    plan = make_plan(w, V, phi, mu=mu)
+    for nvec in (1, 3):
+        x = synth.random_block(w, nvec, seed=31 + nvec)
+        for mode in (bdg.UV, bdg.FG):
+            y = plan.apply(torch.from_numpy(x).cuda(), mode).cpu().numpy()
+            ref = op.apply_fft(x, mode)
+            # about 40 roundings of 2^-53 in a row, relative to the largest symbol times x (y is of its size)
+            assert np.linalg.norm((y - ref).ravel()) < 1e-13 * np.linalg.norm(ref.ravel()), (mode, nvec)
+    many = 5000 * max(n) // (6 * plan.npts) + 1
+    xt = torch.randn((many, 6, plan.npts), dtype=torch.complex128, device="cuda",
+                     generator=torch.Generator(device="cuda").manual_seed(5))
+    for mode in (bdg.UV, bdg.FG):
+        y = plan.apply(xt, mode)
+        one = torch.cat([plan.apply(xt[i:i + 1], mode) for i in (0, many // 2, many - 1)])
+        two = y[[0, many // 2, many - 1]]
+        assert float((one - two).norm() / two.norm()) < 1e-13
+    plan.close()
