@@ -417,14 +417,8 @@ static void free_plan(bdg_plan_t plan) {
   delete plan;
 }
 
-}  // namespace bdg
-
-using namespace bdg;
-
-extern "C" {
-
-bdg_status bdg_plan_create(bdg_plan_t* out, const bdg_params* p, const double* V, const double* phi,
-                           void* stream) {
+bdg_status create_plan(bdg_plan_t* out, const bdg_params* p, const double* V, const double* phi, cudaStream_t s,
+                       bool deflation) {
   if (!out) return fail(nullptr, BDG_ERR_INVALID, "out is NULL");
   *out = nullptr;
   Grid g;
@@ -432,7 +426,6 @@ bdg_status bdg_plan_create(bdg_plan_t* out, const bdg_params* p, const double* V
   bdg_status st = validate(p, &g, &why);
   if (st) return fail(nullptr, st, why);
   if (!V || !phi) return fail(nullptr, BDG_ERR_INVALID, "V and phi must be host pointers");
-  cudaStream_t s = (cudaStream_t)stream;
   bdg_plan_t plan = new (std::nothrow) bdg_plan_s();
   if (!plan) return fail(nullptr, BDG_ERR_NOMEM, "host allocation failed");
   plan->prm = *p;
@@ -500,15 +493,25 @@ bdg_status bdg_plan_create(bdg_plan_t* out, const bdg_params* p, const double* V
     for (int j = 0; j < 3; ++j)
       if (std::isnan(p->mu[j])) plan->mu[j] = mu[j];
   }
-  st = build_deflation(plan, s);
-  if (st) {
+  if (deflation && (st = build_deflation(plan, s))) {
     std::string m = plan->err;
     free_plan(plan);
     return fail(nullptr, st, m);
   }
-  plan->last_stream = stream;
+  plan->last_stream = s;
   *out = plan;
   return BDG_OK;
+}
+
+}  // namespace bdg
+
+using namespace bdg;
+
+extern "C" {
+
+bdg_status bdg_plan_create(bdg_plan_t* out, const bdg_params* p, const double* V, const double* phi,
+                           void* stream) {
+  return create_plan(out, p, V, phi, (cudaStream_t)stream, true);
 }
 
 bdg_status bdg_plan_destroy(bdg_plan_t plan) {

@@ -20,4 +20,9 @@ struct KdArgs {
 template <typename R>
 cudaError_t kdiag_launch(const KdArgs<R>& g);
 
+// y = -1/2 Lap x (eq. laplace_approx) on nplanes planes, x != y (shift and
+// scale are not used)
+template <typename R>
+cudaError_t laplacian_launch(const KdArgs<R>& g);
+
 }  // namespace bdg

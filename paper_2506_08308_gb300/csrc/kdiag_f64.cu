@@ -3,4 +3,5 @@
 
 namespace bdg {
 template cudaError_t kdiag_launch<double>(const KdArgs<double>&);
+template cudaError_t laplacian_launch<double>(const KdArgs<double>&);
 }  // namespace bdg

@@ -16,13 +16,15 @@
 
 namespace bdg {
 
-enum { KD_FWD = 0, KD_INV = 1, KD_FMI = 2 };
+// KD_LAP: forward, 1/2 mu^2 of this axis alone, inverse; the strided passes add to y
+enum { KD_FWD = 0, KD_INV = 1, KD_FMI = 2, KD_LAP = 3 };
 
 struct KdCoef {
   double shift, scale;   // g = 1 / (shift + scale * sum_a kappa_a k_a^2)
   double kappa[3];       // (2 pi / len_a)^2
   int n[3];
   double norm;           // 1 / N_p
+  double lap[3];         // 1/2 kappa_a / n_a
 };
 
 // Contiguous lines (last axis): warp-mapped, 8 warps per CTA.  x may equal y
@@ -73,6 +75,16 @@ __global__ void __launch_bounds__(256) k_kd_contig(const typename CT<R>::T* x,
         b[s][k2] = b[s][k2] * ((R)c.norm / d);
       }
   }
+  if (sizeof(R) == 8 && mode == KD_LAP) {  // (only the FP64 ground state uses it)
+    const R ks = (R)(axis == 0 ? c.lap[0] : axis == 1 ? c.lap[1] : c.lap[2]);
+#pragma unroll
+    for (int s = 0; s < L::S; ++s)
+#pragma unroll
+      for (int k2 = 0; k2 < N1; ++k2) {
+        const int kk = kidx<N>(t + N1 * s + N2 * k2);
+        b[s][k2] = b[s][k2] * (ks * (R)(kk * kk));
+      }
+  }
   if (mode == KD_FWD) {
     L::toNatural(b, t, ex, WarpSync());
 #pragma unroll
@@ -97,7 +109,7 @@ __global__ void __launch_bounds__(W * Split<N>::N1) k_kd_strided(const typename 
                                                                 long long npts, long long st,
                                                                 long long tiles_per_plane,
                                                                 const typename CT<R>::T* __restrict__ twg,
-                                                                int mode, KdCoef c) {
+                                                                int mode, KdCoef c, int axis) {
   typedef typename CT<R>::T T;
   typedef Line<N, T, BlockSync> L;
   constexpr int N1 = L::N1, N2 = L::N2, LS = N + 1;
@@ -153,6 +165,16 @@ __global__ void __launch_bounds__(W * Split<N>::N1) k_kd_strided(const typename 
         b[s][k2] = b[s][k2] * ((R)c.norm / d);
       }
   }
+  if (sizeof(R) == 8 && mode == KD_LAP) {  // (only the FP64 ground state uses it)
+    const R ks = (R)(axis == 0 ? c.lap[0] : c.lap[1]);
+#pragma unroll
+    for (int s = 0; s < L::S; ++s)
+#pragma unroll
+      for (int k2 = 0; k2 < N1; ++k2) {
+        const int kk = kidx<N>(j + N1 * s + N2 * k2);
+        b[s][k2] = b[s][k2] * (ks * (R)(kk * kk));
+      }
+  }
   if (mode == KD_FWD) {
     L::toNatural(b, j, ex, BlockSync());
 #pragma unroll
@@ -162,6 +184,13 @@ __global__ void __launch_bounds__(W * Split<N>::N1) k_kd_strided(const typename 
     L::invA(a, j, ex, tw);
   }
   T* yl = y + base;
+  if (sizeof(R) == 8 && mode == KD_LAP) {
+    T yv[N2];
+#pragma unroll
+    for (int n2 = 0; n2 < N2; ++n2) yv[n2] = yl[(long long)(j + N1 * n2) * st];
+#pragma unroll
+    for (int n2 = 0; n2 < N2; ++n2) a[n2] = a[n2] + yv[n2];
+  }
 #pragma unroll
   for (int n2 = 0; n2 < N2; ++n2) yl[(long long)(j + N1 * n2) * st] = a[n2];
 }
@@ -207,11 +236,23 @@ __global__ void __launch_bounds__(Spread<N, typename CT<R>::T>::FT)
         a[k] = a[k] * ((R)c.norm / (base_d + sk * (R)(kk * kk)));
       }
     }
+    if (mode == KD_LAP) {
+      const R ks = (R)(axis == 0 ? c.lap[0] : axis == 1 ? c.lap[1] : c.lap[2]);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int kk = kidx<N>(t + TH * k);
+        a[k] = a[k] * (ks * (R)(kk * kk));
+      }
+    }
     if (mode != KD_FWD) f.template run<1>(a, t, e, sync);
   };
   if constexpr (FT == 32) go(SpreadWarp());
   else go(SpreadBar<FT>());
   if (act) {
+    if (mode == KD_LAP && st > 1) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) a[k] = a[k] + y[base + TH * k * st];
+    }
 #pragma unroll
     for (int k = 0; k < 4; ++k) y[base + TH * k * st] = a[k];
   }
@@ -270,7 +311,7 @@ static cudaError_t kd_strided_w(const KdArgs<R>& g, const KdCoef& c, int ax, lon
   if (e != cudaSuccess) return e;
   const long long tiles = g.grid->npts / ((long long)N * W);
   kern<<<(unsigned)(tiles * g.nplanes), W * N1, sm, g.stream>>>(x, y, g.grid->npts, st, tiles, g.tw[ax],
-                                                               mode, c);
+                                                               mode, c, ax);
   return cudaGetLastError();
 }
 
@@ -315,8 +356,7 @@ static cudaError_t kd_strided_d(const KdArgs<R>& g, const KdCoef& c, int ax, con
 }
 
 template <typename R>
-cudaError_t kdiag_launch(const KdArgs<R>& g) {
-  if (g.nplanes <= 0) return cudaSuccess;
+static KdCoef kd_coef(const KdArgs<R>& g) {
   KdCoef c;
   c.shift = g.shift;
   c.scale = g.scale;
@@ -324,8 +364,16 @@ cudaError_t kdiag_launch(const KdArgs<R>& g) {
     const double k0 = 2.0 * M_PI / g.grid->len[a];
     c.kappa[a] = k0 * k0;
     c.n[a] = g.grid->n[a];
+    c.lap[a] = 0.5 * c.kappa[a] / c.n[a];
   }
   c.norm = 1.0 / (double)g.grid->npts;
+  return c;
+}
+
+template <typename R>
+cudaError_t kdiag_launch(const KdArgs<R>& g) {
+  if (g.nplanes <= 0) return cudaSuccess;
+  const KdCoef c = kd_coef(g);
   const int d = g.grid->dim;
   cudaError_t e;
   if (d == 1) return kd_contig_d<R>(g, c, g.x, g.y, KD_FMI);
@@ -337,6 +385,15 @@ cudaError_t kdiag_launch(const KdArgs<R>& g) {
   for (int ax = 1; ax <= d - 2; ++ax)
     if ((e = kd_strided_d<R>(g, c, ax, g.y, g.y, KD_INV))) return e;
   return kd_contig_d<R>(g, c, g.y, g.y, KD_INV);
+}
+
+template <typename R>
+cudaError_t laplacian_launch(const KdArgs<R>& g) {
+  if (g.nplanes <= 0) return cudaSuccess;
+  const KdCoef c = kd_coef(g);
+  cudaError_t e = kd_contig_d<R>(g, c, g.x, g.y, KD_LAP);
+  for (int ax = g.grid->dim - 2; e == cudaSuccess && ax >= 0; --ax) e = kd_strided_d<R>(g, c, ax, g.x, g.y, KD_LAP);
+  return e;
 }
 
 }  // namespace bdg

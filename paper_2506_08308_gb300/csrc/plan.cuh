@@ -24,4 +24,9 @@ static_assert(sizeof(bdg_plan_s::scratch) / sizeof(Buffer) == SLOT_COUNT, "one s
 bdg_status apply_internal(bdg_plan_t plan, int mode, int dtype, const void* x, void* y, int nvec,
                           cudaStream_t s, const double* mu_override);
 
+// bdg_plan_create, optionally without the deflation bases (for callers that
+// only use the grid's tables).
+bdg_status create_plan(bdg_plan_t* out, const bdg_params* p, const double* V, const double* phi, cudaStream_t s,
+                       bool deflation);
+
 }  // namespace bdg
