@@ -12,18 +12,29 @@
 // of the two-pass Gram-Schmidt (whose second pass, in double-float, removes
 // what the first one leaves).
 //
+// What bounds it: one CTA used to load, split and multiply each 32-row stage
+// in turn, and waited out a memory latency per stage (48 x 48 columns of
+// 196608 FP64 rows: 288 us, 0.5 TB/s).  Eight or sixteen warps now load
+// and split, two tasks ahead of their use, into a ring of stages, and one
+// more issues the issues the MMAs; the arithmetic and its order are unchanged, bit for bit,
+// and the calls below went from 304 to 90 us (24 x 24 pairs, C128, 196608
+// rows), 194 to 70 (C64), 559 to 363 (72 x 72, C128).  The row chunks, whose
+// number the workspace gives, leave 96 CTAs there: the integer work of cutting
+// FP64 values on those 96 SMs is what bounds it now.
+//
 // Layout of one pipeline stage in shared memory: for A (128 real columns)
-// and B (NT real columns) three BF16 slice tiles of TBK = 32 rows each, in
-// the K-major layout of the MMA without swizzle: core matrices of 8 columns
-// x 8 rows (16 bytes per column), core matrix (k8, c8) at byte offset
-// (k8 * (cols / 8) + c8) * 128.  One MMA step covers 16 rows (two core
-// matrices along K, `lbo` bytes apart; 8-column groups `sbo` = 128 bytes
-// apart).
+// and B (NT real columns) three BF16 slice tiles of TBK = 32 rows each, MN-
+// major without swizzle: a core matrix holds 8 rows of 8 neighbouring real
+// columns (16 bytes a row), core matrix (k8, c8) at byte offset (k8 (cols / 8)
+// + c8) 128.  A warp's task is four complex columns at 32 rows, one row a
+// lane: 512-byte loads, 16-byte stores, no bank conflicts.  One MMA step
+// covers 16 rows (two core matrices along K).
 #include <cuda_bf16.h>
 
 #include <algorithm>
 
 #include "blas.cuh"
+#include "digits.cuh"
 
 namespace bdg {
 
@@ -31,259 +42,201 @@ namespace {
 
 constexpr int TM = 128;          // A real columns per CTA (MMA M)
 constexpr int TBK = 32;          // rows per pipeline stage (two MMA K steps of 16)
-constexpr int TSTAGES = 2;       // stages in flight
-constexpr int TTHREADS = 256;
 constexpr int TNMAX = 160;       // widest B tile (real columns, multiple of 16)
 constexpr int NSLICE = 3;
 constexpr int A_SLICE_BYTES = TM * TBK * 2;
-constexpr long long WAIT_LIMIT = 1LL << 22;  // polls of an MMA barrier before giving up
+// stages in flight, as many as the CTAs of an SM (two with eight producer
+// warps, one with sixteen) have room for
+__host__ __device__ constexpr int stages_of(int NT, int pwarps) { return (NT <= 48 ? 3 : 2) * (pwarps > 8 ? 2 : 1); }
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-// shared-memory matrix descriptor (no swizzle): start address, byte offset
-// between the two core matrices along K, byte offset between 8-column
-// groups, descriptor version 1
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(sbo >> 4) << 32) |
-         (1ull << 46);
-}
-
-// instruction descriptor of kind::f16: D FP32, A and B BF16, both K-major,
-// N >> 3 at bit 17, M >> 4 at bit 24
+// instruction descriptor of kind::f16: D FP32, A and B BF16, both MN-major
 __device__ __forceinline__ uint32_t idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  for (long long it = 0; it < WAIT_LIMIT; ++it) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
-  }
-  return false;
-}
-
-__device__ __forceinline__ uint32_t pack2(__nv_bfloat16 lo, __nv_bfloat16 hi) {
-  return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-}
-
-__device__ __forceinline__ void split3(float x, __nv_bfloat16& a, __nv_bfloat16& b, __nv_bfloat16& c) {
-  a = __float2bfloat16_rn(x);
-  float r = x - __bfloat162float(a);
-  b = __float2bfloat16_rn(r);
-  r -= __bfloat162float(b);
-  c = __float2bfloat16_rn(r);
+  return mma_idesc_f16(M, N, true, true) | (1u << 7) | (1u << 10);
 }
 
 // FP64 x cut to FP32 by its bits (24 significant bits, truncated; below the
 // FP32 normal range 0, above it infinity, NaN kept): no FP64 arithmetic,
 // which runs at a small fraction of the FP32 rate on this part.
 __device__ __forceinline__ float cut_to_float(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const unsigned hi = (unsigned)(b >> 32);
-  const unsigned sign = hi & 0x80000000u;
-  const int ex = (int)((hi >> 20) & 0x7FFu);
-  const unsigned mant = (unsigned)(b >> 29) & 0x7FFFFFu;
-  if (ex == 0x7FF) return __uint_as_float(sign | 0x7F800000u | (mant ? 0x400000u : 0u));
-  const int e = ex - 1023 + 127;
-  if (e <= 0) return __uint_as_float(sign);
-  if (e >= 255) return __uint_as_float(sign | 0x7F800000u);
-  return __uint_as_float(sign | ((unsigned)e << 23) | mant);
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned sign = hi & 0x80000000u, mag = hi & 0x7FFFFFFFu;
+  if (mag - (897u << 20) < (254u << 20))  // exponents 897 .. 1150: the FP32 normal range
+    return __uint_as_float((__funnelshift_l(lo, hi, 3) - (384u << 23)) | sign);  // (896 mod 512) off the 9 bits kept
+  if (mag < (897u << 20)) return __uint_as_float(sign);
+  const bool nan = (mag >> 20) == 0x7FFu && __funnelshift_l(lo, hi, 3) & 0x7FFFFFu;
+  return __uint_as_float(sign | 0x7F800000u | (nan ? 0x400000u : 0u));
 }
+__device__ __forceinline__ float cut_to_float(float x) { return x; }
 
-__device__ __forceinline__ void split3(double x, __nv_bfloat16& a, __nv_bfloat16& b, __nv_bfloat16& c) {
-  split3(cut_to_float(x), a, b, c);
-}
-
-// Rows r .. r+7 of complex column `col` (zero past r_end or past the
-// block's columns) as the slices of real columns c (real parts) and c + 1
-// (imaginary parts) of a tile of `tcols` columns: one 16-byte core-matrix
-// row per slice and real column.
-template <typename R>
-__device__ __forceinline__ void stage_rows(const PairBlock<R>& X, int col, long long r, long long r_end, int c,
-                                           int g, int tcols, uint8_t* base) {
-  typedef typename CT<R>::T T;
-  T v[8];
-  const bool colok = col < X.cols;
-  const T* src = X.p + (long long)(colok ? col : 0) * X.ld + r;
-  if (colok && r + 8 <= r_end && ((uintptr_t)src & 15) == 0) {
-    // whole group in range: 16-byte loads, all in flight together
-    const uint4* s4 = reinterpret_cast<const uint4*>(src);
-    uint4 u[sizeof(T) / 2];
+// the three BF16 slices of two values, packed (first value in the low half)
+__device__ __forceinline__ void split3(float x, float y, uint32_t (&w)[3]) {
 #pragma unroll
-    for (int q = 0; q < (int)(sizeof(T) / 2); ++q) u[q] = __ldg(s4 + q);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = reinterpret_cast<const T*>(u)[q];
-  } else {
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = (colok && r + q < r_end) ? src[q] : mk((R)0, (R)0);
-  }
-  uint32_t w[2][NSLICE][4];
-#pragma unroll
-  for (int q = 0; q < 8; q += 2) {
-    __nv_bfloat16 a0, b0, c0, a1, b1, c1;
-    split3(v[q].x, a0, b0, c0);
-    split3(v[q + 1].x, a1, b1, c1);
-    w[0][0][q / 2] = pack2(a0, a1);
-    w[0][1][q / 2] = pack2(b0, b1);
-    w[0][2][q / 2] = pack2(c0, c1);
-    split3(v[q].y, a0, b0, c0);
-    split3(v[q + 1].y, a1, b1, c1);
-    w[1][0][q / 2] = pack2(a0, a1);
-    w[1][1][q / 2] = pack2(b0, b1);
-    w[1][2][q / 2] = pack2(c0, c1);
-  }
-  const uint32_t slice_bytes = (uint32_t)tcols * TBK * 2;
-  const uint32_t lbo = (uint32_t)(tcols / 8) * 128;
-  // The eight threads of a quarter warp hold eight consecutive complex
-  // columns of one K group: those with complex column % 8 >= 4 store the
-  // imaginary row first, so that every 16-byte store of the quarter warp
-  // lands in a different group of four banks.
-  const int flip = (c >> 3) & 1;
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int part = q ^ flip;
-    const int cc = c + part;
-    const uint32_t off = (uint32_t)g * lbo + (uint32_t)(cc / 8) * 128 + (uint32_t)(cc % 8) * 16;
-#pragma unroll
-    for (int s = 0; s < NSLICE; ++s) {
-      const uint4 u0 = make_uint4(w[0][s][0], w[0][s][1], w[0][s][2], w[0][s][3]);
-      const uint4 u1 = make_uint4(w[1][s][0], w[1][s][1], w[1][s][2], w[1][s][3]);
-      *reinterpret_cast<uint4*>(base + s * slice_bytes + off) = part ? u1 : u0;
+  for (int k = 0; k < 3; ++k) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+    w[k] = *reinterpret_cast<const uint32_t*>(&h);
+    if (k < 2) {
+      x -= __uint_as_float(w[k] << 16);
+      y -= __uint_as_float(w[k] & 0xFFFF0000u);
     }
   }
+}
+
+// Four complex columns of a block at one row (zero past the end).
+template <typename R>
+struct RowTask {
+  typename CT<R>::T v[4];
+};
+template <typename R>
+__device__ __forceinline__ void load_task(const PairBlock<R>& X, int c0, long long r, long long r_end, RowTask<R>& o) {
+  const typename CT<R>::T* p = X.p + (long long)c0 * X.ld + r;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    o.v[q] = mk((R)0, (R)0);
+    if (r < r_end && c0 + q < X.cols) o.v[q] = p[q * X.ld];
+  }
+}
+// slices of eight real columns at one row: 16 bytes per slice tile
+template <typename R>
+__device__ __forceinline__ void store_task(const RowTask<R>& x, uint8_t* base, uint32_t slice_bytes) {
+  uint32_t w[4][NSLICE];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) split3(cut_to_float(x.v[q].x), cut_to_float(x.v[q].y), w[q]);
+#pragma unroll
+  for (int s = 0; s < NSLICE; ++s) *reinterpret_cast<uint4*>(base + s * slice_bytes) = make_uint4(w[0][s], w[1][s], w[2][s], w[3][s]);
 }
 
 // Partial Gram of one row chunk: part[chunk][i][j] for real columns
 // i < 2 A.cols (128 per CTA along x), j < 2 B.cols <= NT.  A wait that runs
 // out writes NaN into the tile (the caller sees a NaN Gram).
-template <typename R>
-__global__ void __launch_bounds__(TTHREADS, 2)
+template <typename R, int PWARPS>
+__global__ void __launch_bounds__(32 * (PWARPS + 1), PWARPS > 8 ? 1 : 2)
     k_gram_tc(PairBlock<R> A, PairBlock<R> B, int NT, long long crows, double* __restrict__ part) {
   extern __shared__ __align__(1024) uint8_t smem[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const int nstage = stages_of(NT, PWARPS);
   const uint32_t b_slice = (uint32_t)NT * TBK * 2;
   const uint32_t stage_bytes = NSLICE * (A_SLICE_BYTES + b_slice);
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(smem + TSTAGES * stage_bytes);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mbar + TSTAGES);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + nstage * stage_bytes);
+  uint64_t* empty = full + nstage;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(empty + nstage);
   const uint32_t ncols = NT <= 32 ? 32u : NT <= 64 ? 64u : NT <= 128 ? 128u : 256u;
   const int i0 = blockIdx.x * TM;
   const long long r_begin = (long long)blockIdx.z * crows;
   const long long r_end = min(A.n, r_begin + crows);
   const int P2 = 2 * A.cols, Q2 = 2 * B.cols;
 
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(ncols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
+  if (warp == PWARPS) tmem_alloc(tmem_slot, ncols);
   if (tid == 0) {
-    for (int s = 0; s < TSTAGES; ++s)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[s])) : "memory");
+    for (int s = 0; s < nstage; ++s) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[s])), "r"(PWARPS) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&empty[s])) : "memory");
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  tc_fence_before();
   __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
   const int nsteps = r_end > r_begin ? (int)((r_end - r_begin + TBK - 1) / TBK) : 0;
   bool lost = false;
-  for (int step = 0; step < nsteps; ++step) {
-    const int st = step % TSTAGES;
-    uint8_t* sa = smem + st * stage_bytes;
-    uint8_t* sb = sa + NSLICE * A_SLICE_BYTES;
-    // the MMAs that read this stage (committed TSTAGES steps ago) are done
-    if (step >= TSTAGES && !mbar_wait(smem_u32(&mbar[st]), (uint32_t)((step / TSTAGES - 1) & 1))) lost = true;
-    const long long r0 = r_begin + (long long)step * TBK;
-    // A: 64 complex columns x 4 groups of 8 rows, one group per thread;
-    // task t -> column (t & 7) + 8 (t >> 5), group (t >> 3) & 3: a quarter
-    // warp covers eight consecutive columns of one group
-    {
-      const int c = (tid & 7) | ((tid >> 5) << 3), g = (tid >> 3) & 3;
-      stage_rows<R>(A, i0 / 2 + c, r0 + 8 * g, r_end, 2 * c, g, TM, sa);
-    }
-    for (int t = tid; t < (NT / 2) * 4; t += TTHREADS) {
-      const int c = (t & 7) | ((t >> 5) << 3), g = (t >> 3) & 3;
-      stage_rows<R>(B, c, r0 + 8 * g, r_end, 2 * c, g, NT, sb);
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t idesc = idesc_bf16(TM, NT);
-      const uint32_t lbo_a = (TM / 8) * 128, lbo_b = (uint32_t)(NT / 8) * 128;
-      // slice pairs (A slice, B slice) whose weight reaches 2^-24 of the leading one
-      const int pa[6] = {0, 0, 1, 1, 0, 2}, pb[6] = {0, 1, 0, 1, 2, 0};
+  if (warp == PWARPS) {
+    const uint32_t idesc = idesc_bf16(TM, NT);
+    const uint32_t lbo_a = (TM / 8) * 128, lbo_b = (uint32_t)(NT / 8) * 128;
+    const bool leader = elect_one();
+    int st = 0, ph = 0;
+    for (int step = 0; step < nsteps; ++step) {
+      if (!mma_wait(&full[st], (uint32_t)ph)) lost = true;
+      tc_fence_after();
+      if (leader) {
+        const uint32_t sa = smem_u32(smem + st * stage_bytes), sb = sa + NSLICE * A_SLICE_BYTES;
+        // slice pairs (A slice, B slice) whose weight reaches 2^-24 of the leading one
+        const int pa[6] = {0, 0, 1, 1, 0, 2}, pb[6] = {0, 1, 0, 1, 2, 0};
 #pragma unroll
-      for (int p = 0; p < 6; ++p)
+        for (int p = 0; p < 6; ++p)
 #pragma unroll
-        for (int kk = 0; kk < 2; ++kk) {
-          const uint64_t ad = sdesc(smem_u32(sa + pa[p] * A_SLICE_BYTES + 2 * kk * lbo_a), lbo_a, 128);
-          const uint64_t bd = sdesc(smem_u32(sb + pb[p] * b_slice + 2 * kk * lbo_b), lbo_b, 128);
-          const uint32_t acc = (step > 0 || p > 0 || kk > 0) ? 1u : 0u;
-          asm volatile(
-              "{\n\t.reg .pred p;\n\t"
-              "setp.ne.b32 p, %4, 0;\n\t"
-              "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-              "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-              : "memory");
-        }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       smem_u32(&mbar[st]))
-                   : "memory");
+          for (int kk = 0; kk < 2; ++kk)
+            mma_f16(tmem, mma_desc(sa + pa[p] * A_SLICE_BYTES + 2 * kk * lbo_a, lbo_a, 128),
+                    mma_desc(sb + pb[p] * b_slice + 2 * kk * lbo_b, lbo_b, 128), idesc, step > 0 || p > 0 || kk > 0);
+        mma_commit(&empty[st]);
+      }
+      __syncwarp();
+      if (++st == nstage) { st = 0; ph ^= 1; }
+    }
+  } else {
+    // tasks of a stage: groups of four complex columns of A, then of B; this
+    // warp takes every PWARPS-th.  Rows of A's tile past the block's columns are
+    // never written: they only reach rows of the result that nothing reads.
+    const int na = (min(TM, P2 - i0) + 7) / 8, nt = na + (Q2 + 7) / 8;
+    const int per = (nt + PWARPS - 1) / PWARPS;
+    // items (step, q) in order, loads two items ahead
+    int fs = 0, fq = 0;
+    auto fetch = [&](RowTask<R>& x) {
+      const int t = warp + PWARPS * fq;
+      const long long r = r_begin + (long long)fs * TBK + lane;
+      if (fs < nsteps) {
+        if (t < na) load_task<R>(A, i0 / 2 + 4 * t, r, r_end, x);
+        else if (t < nt) load_task<R>(B, 4 * (t - na), r, r_end, x);
+      }
+      if (++fq == per) { fq = 0; ++fs; }
+    };
+    int step = 0, q = 0, st = 0, ph = 1;   // (a fresh barrier's other phase counts as complete)
+    auto produce = [&](RowTask<R>& x) {
+      if (step >= nsteps) return;
+      // the MMAs that read this stage nstage steps ago are done
+      if (q == 0 && !mma_wait(&empty[st], (uint32_t)ph)) lost = true;
+      const int t = warp + PWARPS * q;
+      if (t < nt) {
+        uint8_t* base = t < na ? smem + st * stage_bytes + ((lane >> 3) * (TM / 8) + t) * 128
+                               : smem + st * stage_bytes + NSLICE * A_SLICE_BYTES + ((lane >> 3) * (NT / 8) + t - na) * 128;
+        store_task<R>(x, base + (lane & 7) * 16, t < na ? (uint32_t)A_SLICE_BYTES : b_slice);
+      }
+      fetch(x);
+      if (++q == per) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full[st])) : "memory");
+        q = 0;
+        ++step;
+        if (++st == nstage) { st = 0; ph ^= 1; }
+      }
+    };
+    RowTask<R> x0, x1;
+    fetch(x0);
+    fetch(x1);
+    for (int item = 0; item < nsteps * per; item += 2) {
+      produce(x0);
+      produce(x1);
     }
   }
-  if (nsteps > 0) {
-    const int last = nsteps - 1;
-    if (!mbar_wait(smem_u32(&mbar[last % TSTAGES]), (uint32_t)((last / TSTAGES) & 1))) lost = true;
-  }
+  const int last = nsteps - 1;
+  if (nsteps > 0 && !mma_wait(&empty[last % nstage], (uint32_t)((last / nstage) & 1))) lost = true;
   lost = __syncthreads_or(lost) != 0;
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const int quarter = warp & 3;  // a warp reads TMEM lanes 32 quarter .. 32 quarter + 31
-  const int i = i0 + 32 * quarter + lane;
-  double* out = part + (long long)blockIdx.z * P2 * Q2;
-  for (int jc = (warp >> 2) * 16; jc < NT; jc += 32) {
-    uint32_t v[16];
-    if (nsteps > 0) {
-      const uint32_t ta = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)jc;
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-            "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-          : "r"(ta)
-          : "memory");
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    } else {
+  tc_fence_after();
+  if (warp < PWARPS) {
+    const int quarter = warp & 3;  // a warp reads TMEM lanes 32 quarter .. 32 quarter + 31
+    const int i = i0 + 32 * quarter + lane;
+    double* out = part + (long long)blockIdx.z * P2 * Q2;
+    for (int jc = (warp >> 2) * 4; jc < NT; jc += PWARPS) {
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
+      if (nsteps > 0) {
+        tmem_ld4(tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)jc, v);
+        tmem_ld_wait();
+      }
+      if (i < P2) {
 #pragma unroll
-      for (int q = 0; q < 16; ++q) v[q] = 0u;
-    }
-    if (i < P2) {
-#pragma unroll
-      for (int q = 0; q < 16; ++q) {
-        const int j = jc + q;
-        if (j < Q2) out[(long long)i * Q2 + j] = lost ? (double)NAN : (double)__uint_as_float(v[q]);
+        for (int q = 0; q < 4; ++q)
+          if (jc + q < Q2) out[(long long)i * Q2 + jc + q] = lost ? (double)NAN : (double)v[q];
       }
     }
   }
   if (lost && nsteps > 0) {
     // the MMAs may still run: wait (bounded) for the last commit before freeing their accumulator
-    const int last = nsteps - 1;
-    mbar_wait(smem_u32(&mbar[last % TSTAGES]), (uint32_t)((last / TSTAGES) & 1));
+    mma_wait(&empty[last % nstage], (uint32_t)((last / nstage) & 1));
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  tc_fence_before();
   __syncthreads();
-  if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
+  if (warp == PWARPS) tmem_free(tmem, ncols);
 }
 
 // G[e] = sum over chunks, in a fixed order: thread (x, y) of a 32 x 8 block
@@ -308,8 +261,9 @@ __global__ void __launch_bounds__(256) k_gram_tc_reduce(const double* __restrict
   }
 }
 
-size_t tc_smem_bytes(int NT) {
-  return (size_t)TSTAGES * NSLICE * (A_SLICE_BYTES + (size_t)NT * TBK * 2) + 8 * TSTAGES + 16;
+size_t tc_smem_bytes(int NT, int pwarps) {
+  const int n = stages_of(NT, pwarps);
+  return (size_t)n * NSLICE * (A_SLICE_BYTES + (size_t)NT * TBK * 2) + 16 * n + 16;
 }
 
 }  // namespace
@@ -329,15 +283,18 @@ cudaError_t gram_pairs_tc(const PairBlock<R>& A, const PairBlock<R>& B, double* 
   const size_t per_chunk = sizeof(double) * (size_t)P2 * Q2;
   const long long cap = (long long)(ws_bytes / per_chunk);
   if (cap < 1) return cudaErrorInvalidValue;
-  // about two CTAs per SM (each holds two stages and 32 ... 256 TMEM columns)
+  // two CTAs per SM (each holds two or three stages and 32 ... 256 TMEM columns)
   long long nch = std::min<long long>((2 * 152 + mtiles - 1) / mtiles, cap);
   nch = std::min<long long>(nch, (A.n + TBK - 1) / TBK);
   const long long crows = ((A.n + nch - 1) / nch + TBK - 1) / TBK * TBK;
   nch = (A.n + crows - 1) / crows;
-  const size_t smem = tc_smem_bytes(NT);
-  cudaError_t e = allow_dynamic_smem((const void*)k_gram_tc<R>, smem);
+  // few row chunks leave an SM with one CTA: then sixteen producer warps
+  const bool wide = nch * mtiles <= 152;
+  const size_t smem = tc_smem_bytes(NT, wide ? 16 : 8);
+  auto kern = wide ? k_gram_tc<R, 16> : k_gram_tc<R, 8>;
+  cudaError_t e = allow_dynamic_smem((const void*)kern, smem);
   if (e != cudaSuccess) return e;
-  k_gram_tc<R><<<dim3((unsigned)mtiles, 1, (unsigned)nch), TTHREADS, smem, s>>>(A, B, NT, crows, (double*)ws);
+  kern<<<dim3((unsigned)mtiles, 1, (unsigned)nch), 32 * (wide ? 17 : 9), smem, s>>>(A, B, NT, crows, (double*)ws);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const int nout = P2 * Q2;
   k_gram_tc_reduce<<<(nout + 31) / 32, 256, 0, s>>>((const double*)ws, (int)nch, nout, G_dev);
