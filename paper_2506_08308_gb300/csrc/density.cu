@@ -40,12 +40,26 @@ __device__ __forceinline__ void load_phi(const float4* __restrict__ p, long long
 constexpr int INLINE_PHASES = 128;
 template <typename C> struct InlinePhases { C v[INLINE_PHASES]; };
 
-// blockIdx.y = mode l; a grid-stride loop over the points.  Entry l * nt + t
-// of the phase table (ph, or inl when ph is NULL) holds
+// V neighbouring complex values / reals in one access
+template <typename R, int V> struct Pack;
+template <> struct Pack<float, 1> { typedef float2 C; typedef float O; };
+template <> struct Pack<float, 2> { typedef float4 C; typedef float2 O; };
+template <> struct Pack<double, 1> { typedef double2 C; typedef double O; };
+__device__ __forceinline__ void unpack(float2 v, float2 (&o)[1]) { o[0] = v; }
+__device__ __forceinline__ void unpack(double2 v, double2 (&o)[1]) { o[0] = v; }
+__device__ __forceinline__ void unpack(float4 v, float2 (&o)[2]) { o[0] = make_float2(v.x, v.y); o[1] = make_float2(v.z, v.w); }
+__device__ __forceinline__ float pack(const float (&o)[1]) { return o[0]; }
+__device__ __forceinline__ double pack(const double (&o)[1]) { return o[0]; }
+__device__ __forceinline__ float2 pack(const float (&o)[2]) { return make_float2(o[0], o[1]); }
+
+// blockIdx.y = mode l; a grid-stride loop over groups of V points.  Entry l *
+// nt + t of the phase table (ph, or inl when ph is NULL) holds
 // (eps cos w_l t, eps sin w_l t), formed in FP64 and rounded to R (an FP32
 // kernel that converted FP64 phases per point would keep the slow FP64 pipe
-// busy); out is [nmode][nt][3][np].
-template <typename R>
+// busy); out is [nmode][nt][3][np].  The amplitudes are read once and the
+// densities written once, past L1 (streaming): with V = 2 a thread has six
+// 16-byte loads in flight where it had six of 8 bytes.
+template <typename R, int V>
 __global__ void __launch_bounds__(256) k_perturbed_density(long long np, int nt,
                                                            const typename CT<R>::T* __restrict__ uv,
                                                            const typename CT<R>::Q* __restrict__ phiv,
@@ -53,22 +67,33 @@ __global__ void __launch_bounds__(256) k_perturbed_density(long long np, int nt,
                                                            const __grid_constant__ InlinePhases<typename CT<R>::T> inl,
                                                            R* __restrict__ out) {
   typedef typename CT<R>::T C;
+  typedef typename Pack<R, V>::C PC;
+  typedef typename Pack<R, V>::O PO;
   const long long l = blockIdx.y;
   const C* x = uv + l * 6 * np;
   const C* pl = ph ? ph + l * nt : nullptr;
   const int i0 = (int)l * nt;
   R* o = out + l * nt * 3 * np;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < np;
-       i += (long long)gridDim.x * blockDim.x) {
-    R f[3], a[3], b[3], d[3], e[3];
-    load_phi(phiv, i, f);
+  for (long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * V; i < np;
+       i += (long long)gridDim.x * blockDim.x * V) {
+    PC z[6];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) z[j] = __ldcs(reinterpret_cast<const PC*>(x + j * np + i));
+    R f[V][3], a[3][V], b[3][V], d[3][V], e[3][V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) load_phi(phiv, i + v, f[v]);
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      const C u = x[j * np + i], v = x[(3 + j) * np + i];
-      a[j] = u.x + v.x;
-      b[j] = u.y + v.y;
-      d[j] = u.y - v.y;
-      e[j] = v.x - u.x;
+      C u[V], w[V];
+      unpack(z[j], u);
+      unpack(z[3 + j], w);
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        a[j][v] = u[v].x + w[v].x;
+        b[j][v] = u[v].y + w[v].y;
+        d[j][v] = u[v].y - w[v].y;
+        e[j][v] = w[v].x - u[v].x;
+      }
     }
     for (int t = 0; t < nt; ++t) {
       const C cs = pl ? pl[t] : inl.v[i0 + t];
@@ -76,10 +101,15 @@ __global__ void __launch_bounds__(256) k_perturbed_density(long long np, int nt,
       R* ot = o + (long long)t * 3 * np + i;
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
-        const R re = fma(a[j], c, b[j] * s);
-        const R im = fma(d[j], c, e[j] * s);
-        const R y = f[j] + re;
-        ot[j * np] = fma(y, y, im * im);
+        R n[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+          const R re = fma(a[j][v], c, b[j][v] * s);
+          const R im = fma(d[j][v], c, e[j][v] * s);
+          const R y = f[v][j] + re;
+          n[v] = fma(y, y, im * im);
+        }
+        __stcs(reinterpret_cast<PO*>(ot + j * np), pack(n));
       }
     }
   }
@@ -129,7 +159,9 @@ extern "C" bdg_status bdg_perturbed_density(bdg_plan_t plan, int dtype, const vo
     if (st) return st;
     ph = plan->scratch[SLOT_PHASE].ptr;
   }
-  long long gx = (np + 255) / 256;
+  // two points per access where both arrays allow it (np is a power of two, at least 8)
+  const bool two = dtype == BDG_C64 && (uintptr_t)UV % 16 == 0 && (uintptr_t)out % 8 == 0;
+  long long gx = (np / (two ? 2 : 1) + 255) / 256;
   const long long cap = 4 * 152 * 8 / nmode + 1;   // about four waves of 8 resident 256-thread CTAs per SM
   if (gx > cap) gx = cap;
   const dim3 grid((unsigned)gx, (unsigned)nmode);
@@ -142,7 +174,7 @@ extern "C" bdg_status bdg_perturbed_density(bdg_plan_t plan, int dtype, const vo
     } else {
       BDG_CUDA_TRY(plan, cudaMemcpyAsync(ph, tab.data(), sizeof(double2) * tab.size(), cudaMemcpyHostToDevice, s));
     }
-    k_perturbed_density<double><<<grid, 256, 0, s>>>(np, nt, (const double2*)UV, plan->phiv64, (const double2*)ph,
+    k_perturbed_density<double, 1><<<grid, 256, 0, s>>>(np, nt, (const double2*)UV, plan->phiv64, (const double2*)ph,
                                                      inl, (double*)out);
   } else {
     std::vector<float2> tab32(tab.size());
@@ -153,8 +185,8 @@ extern "C" bdg_status bdg_perturbed_density(bdg_plan_t plan, int dtype, const vo
     } else {
       BDG_CUDA_TRY(plan, cudaMemcpyAsync(ph, tab32.data(), sizeof(float2) * tab32.size(), cudaMemcpyHostToDevice, s));
     }
-    k_perturbed_density<float><<<grid, 256, 0, s>>>(np, nt, (const float2*)UV, plan->phiv32, (const float2*)ph,
-                                                    inl, (float*)out);
+    auto kern = two ? k_perturbed_density<float, 2> : k_perturbed_density<float, 1>;
+    kern<<<grid, 256, 0, s>>>(np, nt, (const float2*)UV, plan->phiv32, (const float2*)ph, inl, (float*)out);
   }
   BDG_CUDA_TRY(plan, cudaGetLastError());
   plan->last_stream = stream;
