@@ -81,7 +81,8 @@ def load() -> ctypes.CDLL:
     lib.bdg_ground_state.argtypes = [ctypes.POINTER(Params), ctypes.c_double, dp, dp, ctypes.c_double,
                                      ctypes.c_int, dp, dp, dp, ip, vp]
     lib.bdg_chemical_potentials_noalloc.argtypes = [vp, dp, vp]
-    lib.bdg_perturbed_density.argtypes = [vp, ctypes.c_int, vp, ctypes.c_int, dp, dp, ctypes.c_int,
+    # (host arrays as addresses, which a numpy array gives faster than a typed pointer)
+    lib.bdg_perturbed_density.argtypes = [vp, ctypes.c_int, vp, ctypes.c_int, vp, vp, ctypes.c_int,
                                           ctypes.c_double, vp, vp]
     lib.bdg_gram.argtypes = [ctypes.c_int, ctypes.c_int, vp, ctypes.c_longlong, ctypes.c_int, vp,
                              ctypes.c_longlong, ctypes.c_int, ctypes.c_longlong, vp, vp]
@@ -94,15 +95,34 @@ def load() -> ctypes.CDLL:
     return lib
 
 
-def _stream_handle(stream) -> ctypes.c_void_p:
-    """The cudaStream_t of a torch stream; None -> torch's current stream
-    (NULL, the legacy default stream, when torch sees no CUDA device)."""
-    import torch
+_torch = None   # the torch module and its complex dtypes' codes, once a call has needed them
+_CODES = {}
+_raw_stream = None
+
+
+def _get_torch():
+    global _torch, _raw_stream
+    if _torch is None:
+        import torch
+        _CODES.update({torch.complex128: C128, torch.complex64: C64})
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        _torch = torch
+    return _torch
+
+
+def _stream_handle(stream):
+    """The cudaStream_t (an address, or None) of a torch stream; None -> torch's
+    current stream (NULL, the legacy default stream, when torch sees no CUDA
+    device)."""
+    torch = _get_torch()
     if stream is None:
+        if _raw_stream is not None and torch.cuda.is_initialized():
+            # the current stream of the current device, without a Stream object for it
+            return _raw_stream(torch._C._cuda_getDevice()) or None
         if not torch.cuda.is_available():
-            return ctypes.c_void_p(None)
+            return None
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    return stream.cuda_stream or None
 
 
 def _ptr(t) -> ctypes.c_void_p:
@@ -202,19 +222,22 @@ class Plan:
 
     def apply(self, x, mode: int = UV, out=None, stream=None):
         """y = M x for a CUDA tensor x of shape (nvec, 6, N_p), complex64/128."""
-        import torch
-        if not x.is_cuda or x.dim() != 3 or x.shape[1] != 6 or x.shape[2] != self.npts:
+        torch = _get_torch()
+        shape = x.shape
+        if not x.is_cuda or len(shape) != 3 or shape[1] != 6 or shape[2] != self.npts:
             raise ValueError("x must be a CUDA tensor of shape (nvec, 6, N_p)")
-        dt = {torch.complex128: C128, torch.complex64: C64}.get(x.dtype)
+        dt = _CODES.get(x.dtype)
         if dt is None:
             raise ValueError("x must be complex64 or complex128")
         x = x.contiguous()
         if out is None:
             out = torch.empty_like(x)
-        _check_out(out, x.shape, x.dtype, x.device)
-        st = self.lib.bdg_apply(self.handle, int(mode), dt, _ptr(x), _ptr(out), int(x.shape[0]),
+        else:
+            _check_out(out, shape, x.dtype, x.device)
+        st = self.lib.bdg_apply(self.handle, int(mode), dt, x.data_ptr(), out.data_ptr(), shape[0],
                                 _stream_handle(stream))
-        _check(self.lib, st, self.handle)
+        if st != OK:
+            _check(self.lib, st, self.handle)
         return out
 
     def perturbed_density(self, UV, omega, times, eps: float, out=None, stream=None):
@@ -222,10 +245,10 @@ class Plan:
         conj(v_j^l) e^{i w_l t})|^2 for a CUDA tensor UV of shape (nmode, 6, N_p)
         (complex128 -> float64 result, complex64 -> float32), shape
         (nmode, nt, 3, N_p)."""
-        import torch
+        torch = _get_torch()
         if not UV.is_cuda or UV.dim() != 3 or UV.shape[1] != 6 or UV.shape[2] != self.npts:
             raise ValueError("UV must be a CUDA tensor of shape (nmode, 6, N_p)")
-        dt = {torch.complex128: C128, torch.complex64: C64}.get(UV.dtype)
+        dt = _CODES.get(UV.dtype)
         if dt is None:
             raise ValueError("UV must be complex64 or complex128")
         UV = UV.contiguous()
@@ -235,12 +258,16 @@ class Plan:
         if om.size != nmode:
             raise ValueError("omega needs one value per mode")
         rdt = torch.float64 if dt == C128 else torch.float32
+        shape = (nmode, ts.size, 3, self.npts)
         if out is None:
-            out = torch.empty((nmode, ts.size, 3, self.npts), device=UV.device, dtype=rdt)
-        _check_out(out, (nmode, ts.size, 3, self.npts), rdt, UV.device)
-        st = self.lib.bdg_perturbed_density(self.handle, dt, _ptr(UV), nmode, _dptr(om), _dptr(ts), int(ts.size),
-                                            float(eps), _ptr(out), _stream_handle(stream))
-        _check(self.lib, st, self.handle)
+            out = torch.empty(shape, device=UV.device, dtype=rdt)
+        else:
+            _check_out(out, shape, rdt, UV.device)
+        st = self.lib.bdg_perturbed_density(self.handle, dt, UV.data_ptr(), nmode, om.__array_interface__["data"][0],
+                                            ts.__array_interface__["data"][0], ts.size, float(eps), out.data_ptr(),
+                                            _stream_handle(stream))
+        if st != OK:
+            _check(self.lib, st, self.handle)
         return out
 
     def biortho(self, F, G, Fl=None, Gl=None, stream=None):
@@ -293,9 +320,9 @@ def gram(A, B, engine: int = GRAM_TENSOR, out=None, stream=None):
     """bdg_gram: G = A^T B over real columns of two blocks of complex columns
     (torch complex64 or complex128 tensors of shape (ncol, n), contiguous
     rows, same dtype and device); G has shape (2 ncol_a, 2 ncol_b), FP64."""
-    import torch
+    torch = _get_torch()
     lib = load()
-    if A.dtype != B.dtype or A.dtype not in (torch.complex64, torch.complex128):
+    if A.dtype != B.dtype or A.dtype not in _CODES:
         raise ValueError("A and B must both be complex64 or both complex128")
     if A.dim() != 2 or B.dim() != 2 or A.shape[1] != B.shape[1]:
         raise ValueError("A and B must be (ncol, n) with the same n")
@@ -308,8 +335,7 @@ def gram(A, B, engine: int = GRAM_TENSOR, out=None, stream=None):
         out = torch.empty(shape, dtype=torch.float64, device=A.device)
     else:
         _check_out(out, shape, torch.float64, A.device)
-    dtype = C64 if A.dtype == torch.complex64 else C128
-    st = lib.bdg_gram(dtype, int(engine), _ptr(A), A.stride(0), A.shape[0], _ptr(B), B.stride(0), B.shape[0],
+    st = lib.bdg_gram(_CODES[A.dtype], int(engine), _ptr(A), A.stride(0), A.shape[0], _ptr(B), B.stride(0), B.shape[0],
                       A.shape[1], _ptr(out), _stream_handle(stream))
     _check(lib, st)
     return out

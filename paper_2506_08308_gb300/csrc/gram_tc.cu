@@ -7,16 +7,15 @@
 // reaches 2^-24 of the leading one are accumulated in FP32 by the MMA:
 // x0 y0, x0 y1, x1 y0, x1 y1, x0 y2, x2 y0.  Each CTA sums a chunk of rows
 // this way and writes its FP32 tile as FP64 partial sums; the chunks are
-// summed in FP64.  The result has FP32 accuracy (a few 2^-24 of
-// sum |a_k b_k|): it serves the Grams of the FP32 phase and the first pass
-// of the two-pass Gram-Schmidt (whose second pass, in double-float, removes
-// what the first one leaves).
+// summed in FP64.  The result has FP32 accuracy: about 1e-6 to 1e-5 of sum
+// |a_k b_k|, most of it the truncation of the tensor cores' FP32 sums.  (The
+// solver's Grams of this accuracy come from digits, gram_digits.cu.)
 //
 // What bounds it: one CTA used to load, split and multiply each 32-row stage
 // in turn, and waited out a memory latency per stage (48 x 48 columns of
 // 196608 FP64 rows: 288 us, 0.5 TB/s).  Eight or sixteen warps now load
 // and split, two tasks ahead of their use, into a ring of stages, and one
-// more issues the issues the MMAs; the arithmetic and its order are unchanged, bit for bit,
+// more issues the MMAs; the arithmetic and its order are unchanged, bit for bit,
 // and the calls below went from 304 to 90 us (24 x 24 pairs, C128, 196608
 // rows), 194 to 70 (C64), 559 to 363 (72 x 72, C128).  The row chunks, whose
 // number the workspace gives, leave 96 CTAs there: the integer work of cutting
