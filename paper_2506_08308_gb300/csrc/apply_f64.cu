@@ -24,13 +24,32 @@ static cudaError_t axis_spread(const ApplyArgs<R>& g, int ax, cudaStream_t s) {
   BDG_DISPATCH_N(g.grid->n[ax], launch_axis_spread, g, ax, s)
 }
 
+// Axes of 128 and 256 points go to the tensor cores from 2048 lines on (64
+// tiles of 32; apply_digits.cu).  Measured per product, before -> digits:
+// 256^2 x 32 UV 3097 -> 995 us, x 48 FG 4414 -> 1312, x 4 435 -> 162 (full
+// FFTs); x 2 (3072 lines) 226 -> 150, 128^2 x 4 114 -> 75 (spread FFTs);
+// 256^2 x 1 (1536 lines) 119, with digits 145: a tile takes 30 (N = 128) or 60
+// us whether or not every SM has one.
+constexpr long long DIGIT_LINES = 2048;
+static bool digits(const ApplyArgs<R>& g, int ax) {
+  return g.kdig[ax] && g.grid->npts / g.grid->n[ax] * 6 * g.nvec > DIGIT_LINES;
+}
+
 template <>
 cudaError_t apply_launch<double>(const ApplyArgs<double>& g, cudaStream_t s) {
   if (g.nvec <= 0) return cudaSuccess;
   const int last = g.grid->dim - 1;
-  cudaError_t e = few_lines(g, g.grid->n[last]) ? row_spread(g, s) : row_full(g, s);
-  for (int ax = last - 1; e == cudaSuccess && ax >= 0; --ax)
-    e = few_lines(g, g.grid->n[ax]) ? axis_spread(g, ax, s) : axis_full(g, ax, s);
+  cudaError_t e;
+  if (digits(g, last)) {
+    e = couple_launch(g, s);
+    if (e == cudaSuccess) e = axis_digits_launch(g, last, s);
+  } else {
+    e = few_lines(g, g.grid->n[last]) ? row_spread(g, s) : row_full(g, s);
+  }
+  for (int ax = last - 1; e == cudaSuccess && ax >= 0; --ax) {
+    if (digits(g, ax)) e = axis_digits_launch(g, ax, s);
+    else e = few_lines(g, g.grid->n[ax]) ? axis_spread(g, ax, s) : axis_full(g, ax, s);
+  }
   return e;
 }
 

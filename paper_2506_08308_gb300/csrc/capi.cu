@@ -145,6 +145,9 @@ static ApplyArgs<R> make_args(bdg_plan_t plan, int mode, const void* x, void* y,
     g.tw[a] = (const typename CT<R>::T*)(sizeof(R) == 8 ? (const void*)plan->tw64[a] : (const void*)plan->tw32[a]);
     const double k0 = 2.0 * M_PI / plan->grid.len[a];
     g.kscale[a] = (R)(0.5 * k0 * k0 / plan->grid.n[a]);
+    g.kfac[a] = 0.5 * k0 * k0;
+    g.kdig[a] = plan->kdig[a];
+    g.kexp[a] = plan->kexp[a];
   }
   const bdg_params& p = plan->prm;
   g.cp.beta_n = (R)p.beta_n;
@@ -408,6 +411,7 @@ static void free_plan(bdg_plan_t plan) {
   for (int a = 0; a < 3; ++a) {
     cudaFree(plan->tw64[a]);
     cudaFree(plan->tw32[a]);
+    cudaFree(plan->kdig[a]);
   }
   cudaFree(plan->zf64);
   cudaFree(plan->zg64);
@@ -470,6 +474,7 @@ bdg_status create_plan(bdg_plan_t* out, const bdg_params* p, const double* V, co
     CREATE_TRY(cudaMalloc(&plan->tw32[a], sizeof(float2) * g.n[a]));
     CREATE_TRY(cudaMemcpyAsync(plan->tw64[a], t64.data(), sizeof(double2) * g.n[a], cudaMemcpyHostToDevice, s));
     CREATE_TRY(cudaMemcpyAsync(plan->tw32[a], t32.data(), sizeof(float2) * g.n[a], cudaMemcpyHostToDevice, s));
+    if (deflation && axis_digits_supported(g.n[a])) CREATE_TRY(axis_digits_table(g.n[a], &plan->kdig[a], &plan->kexp[a], s));
   }
   CREATE_TRY(cudaStreamSynchronize(s));
 #undef CREATE_TRY

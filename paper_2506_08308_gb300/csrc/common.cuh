@@ -98,6 +98,8 @@ struct bdg_plan_s {
   float4* phiv32 = nullptr;    // the same rounded to FP32
   double2* tw64[3] = {nullptr, nullptr, nullptr};  // W_N^r = exp(-2 pi i r / N), r < N
   float2* tw32[3] = {nullptr, nullptr, nullptr};
+  uint8_t* kdig[3] = {nullptr, nullptr, nullptr};  // digit tables of axes of 128 and 256 points (apply_digits.cu)
+  int kexp[3] = {0, 0, 0};
   // deflation bases (orthonormal columns, real, [ncol][3][N_p] FP64 and FP32)
   int nzf = 0, nzg = 0;
   double* zf64 = nullptr;
