@@ -60,6 +60,15 @@ template <typename R>
 cudaError_t update_pairs(const PairBlock<R>& A, const double* C_dev, int ldc, double beta,
                          typename CT<R>::T* Y, long long ldy, int Q, cudaStream_t s, double alpha = 1.0);
 
+// The same for FP64 blocks from exact integer digits on the tensor cores
+// (update_digits.cu); ws must hold update_digits_workspace_bytes().  Rows of A
+// are rounded to 2^-55 of their largest value: for coefficients that do not
+// make up for columns of A of very different size (no selections of columns).
+size_t update_digits_workspace_bytes();
+bool update_digits_pays(int P, int Q, long long n);
+cudaError_t update_pairs_digits(const PairBlock<double>& A, const double* C_dev, int ldc, double beta, double2* Y,
+                                long long ldy, int Q, void* ws, cudaStream_t s, double alpha = 1.0);
+
 // Y = convert(X) column by column (FP64 <-> FP32 or same type), n complex
 // elements per column, cols columns.
 template <typename RI, typename RO>

@@ -209,6 +209,41 @@ unsigned nblk(long long total) {
   return (unsigned)(b < 1 ? 1 : b);
 }
 
+struct ColumnList {
+  static constexpr int MAX = 64;
+  int c[MAX];
+};
+// out pair q = (real column l.c[2q], l.c[2q + 1]) of the pair bank A; -1: zeros
+template <typename R>
+__global__ void __launch_bounds__(256) k_gather_columns(const typename CT<R>::T* __restrict__ A, long long vlen,
+                                                        const __grid_constant__ ColumnList l,
+                                                        typename CT<R>::T* __restrict__ out) {
+  const int a = l.c[2 * blockIdx.y], b = l.c[2 * blockIdx.y + 1];
+  const typename CT<R>::T *pa = A + (long long)(a < 0 ? 0 : a / 2) * vlen, *pb = A + (long long)(b < 0 ? 0 : b / 2) * vlen;
+  typename CT<R>::T* o = out + (long long)blockIdx.y * vlen;
+  for (long long r = (long long)blockIdx.x * 256 + threadIdx.x; r < vlen; r += (long long)gridDim.x * 256) {
+    const typename CT<R>::T u = pa[r], v = pb[r];
+    o[r] = mk(a < 0 ? (R)0 : a & 1 ? u.y : u.x, b < 0 ? (R)0 : b & 1 ? v.y : v.x);
+  }
+}
+struct ColumnScales {
+  double w[ColumnList::MAX];
+};
+// residuals R_f = HF - G w, R_g = HG - F w of the pairs of (X, HX), column c
+// of the block scaled by s.w[c]
+template <typename R>
+__global__ void __launch_bounds__(256) k_residual(const typename CT<R>::T* __restrict__ X,
+                                                  const typename CT<R>::T* __restrict__ HX, long long n3,
+                                                  const __grid_constant__ ColumnScales s,
+                                                  typename CT<R>::T* __restrict__ out) {
+  const R wx = (R)s.w[2 * blockIdx.y], wy = (R)s.w[2 * blockIdx.y + 1];
+  const long long off = (long long)blockIdx.y * 2 * n3;
+  for (long long r = (long long)blockIdx.x * 256 + threadIdx.x; r < 2 * n3; r += (long long)gridDim.x * 256) {
+    const typename CT<R>::T h = HX[off + r], x = X[off + (r < n3 ? r + n3 : r - n3)];
+    out[off + r] = mk(fma(-wx, x.x, h.x), fma(-wy, x.y, h.y));
+  }
+}
+
 // ---------------------------------------------------------------------------
 // host-side helpers for small matrices
 // ---------------------------------------------------------------------------
@@ -218,7 +253,6 @@ struct HostMat {
   HostMat() {}
   HostMat(int r_, int c_) : r(r_), c(c_), a((size_t)r_ * c_, 0.0) {}
   double& operator()(int i, int j) { return a[(size_t)i * c + j]; }
-  double operator()(int i, int j) const { return a[(size_t)i * c + j]; }
 };
 
 }  // namespace
@@ -360,8 +394,26 @@ class Solver {
   bdg_status update_dev(const PairBlock<R>& A, const double* dC, int ldc, double beta, T* y, int Q,
                         double alpha = 1.0) {
     if (Q == 0) return BDG_OK;
+    if constexpr (sizeof(R) == 8) {
+      plan_->stats.flops_update_df += 2.0 * (double)A.n * (2.0 * A.cols) * (2.0 * Q);
+      if (tc_ && update_digits_pays(A.cols, Q, A.n) && gws_bytes_ >= update_digits_workspace_bytes()) {
+        // (the Gram workspace of the lane is free between its Grams)
+        BDG_CUDA_TRY(plan_, update_pairs_digits(A, dC, ldc, beta, y, vlen_, Q, gws_, s_, alpha));
+        return BDG_OK;
+      }
+    }
     BDG_CUDA_TRY(plan_, update_pairs<R>(A, dC, ldc, beta, y, vlen_, Q, s_, alpha));
-    if (sizeof(R) == 8) plan_->stats.flops_update_df += 2.0 * (double)A.n * (2.0 * A.cols) * (2.0 * Q);
+    return BDG_OK;
+  }
+  // Y (whole 6-component pair columns): real column jj of Y = column sel[jj] of
+  // the bank A; the rest of the nap pairs zero
+  bdg_status gather(const T* A, const std::vector<int>& sel, T* Y, int pairs) {
+    if (pairs == 0) return BDG_OK;
+    if (pairs > ColumnList::MAX / 2 || sel.size() > 2 * (size_t)pairs) return fail(plan_, BDG_ERR_INVALID, "column list too long");
+    ColumnList l;
+    for (int c = 0; c < 2 * pairs; ++c) l.c[c] = c < (int)sel.size() ? sel[c] : -1;
+    k_gather_columns<R><<<dim3(nblk(vlen_), pairs), 256, 0, s_>>>(A, vlen_, l, Y);
+    BDG_CUDA_TRY(plan_, cudaGetLastError());
     return BDG_OK;
   }
   // the same with a host matrix (small data-movement matrices: diagonals, selections)
@@ -891,11 +943,13 @@ class Solver {
       int si_res;
       cudaEvent_t se_res = sec_begin("residuals", &si_res);
       // residuals R_f = HF - G w, R_g = HG - F w
-      BDG_CUDA_TRY(plan_, cudaMemcpyAsync(Rb_, HX, sizeof(T) * vlen_ * mmp, cudaMemcpyDeviceToDevice, s_));
-      HostMat Dw(2 * mmp, 2 * mmp);
-      for (int j = 0; j < mm; ++j) Dw(j, j) = -om[j];
-      if ((st = update(gpart(X, 0, mmp), Dw, 1.0, fptr(Rb_, 0), mmp))) return st;
-      if ((st = update(fpart(X, 0, mmp), Dw, 1.0, gptr(Rb_, 0), mmp))) return st;
+      {
+        if (2 * mmp > ColumnList::MAX) return fail(plan_, BDG_ERR_UNSUPPORTED, "block wider than the residual kernel's list");
+        ColumnScales w = {};
+        for (int j = 0; j < mm; ++j) w.w[j] = om[j];
+        k_residual<R><<<dim3(nblk(vlen_), mmp), 256, 0, s_>>>(X, HX, n3_, w, Rb_);
+        BDG_CUDA_TRY(plan_, cudaGetLastError());
+      }
       // components of G along Z_f (and F along Z_g) in closed form:
       // G += Z_f (Z_f^T R_f) / w, R_f -= Z_f (Z_f^T R_f)
       for (int side = 0; side < 2; ++side) {
@@ -993,9 +1047,7 @@ class Solver {
         for (int jj = 0; jj < na; ++jj) fprintf(stderr, " (%.3e %.3e)", std::sqrt(ng[jj]), std::sqrt(np_[act[jj]]));
         fprintf(stderr, "\n");
       }
-      HostMat Sel(2 * mmp, 2 * nap);
-      for (int jj = 0; jj < na; ++jj) Sel(act[jj], jj) = 1.0;
-      if ((st = update_full(Rb_, mmp, Sel, Wb_, nap))) return st;
+      if ((st = gather(Rb_, act, Wb_, nap))) return st;
       // The previous-update block P (gathered into the second half of W,
       // Gram-Schmidt against X, bi-orthonormalized behind X) does not depend
       // on the new directions: with exact images it runs on the second lane
@@ -1020,11 +1072,8 @@ class Solver {
             if (npn[j] >= 1e-24 * nx[j]) actp.push_back(j);
           const int npa = (int)actp.size();
           if (npa > 0) {
-            HostMat SelP(2 * mmp, 2 * nap);
-            for (int jj = 0; jj < npa; ++jj) SelP(actp[jj], jj) = 1.0;
-            if ((sp = update_full(Pb_, mmp, SelP, Wb_ + (long long)nap * vlen_, nap))) return sp;
-            if (!exact_images_ && (sp = update_full(HPb_, mmp, SelP, HWb_ + (long long)nap * vlen_, nap)))
-              return sp;
+            if ((sp = gather(Pb_, actp, Wb_ + (long long)nap * vlen_, nap))) return sp;
+            if (!exact_images_ && (sp = gather(HPb_, actp, HWb_ + (long long)nap * vlen_, nap))) return sp;
             nw = 4 * nap;
           }
         }
@@ -1119,12 +1168,6 @@ class Solver {
       if (HW && (st = update_dev(gpart(HBk, 0, bp), c2, nw, 1.0, gptr(HW, 0), wp, -1.0))) return st;
     }
     return BDG_OK;
-  }
-
-  // Y (Q pairs) = bank A (P pairs, whole 6-component vectors) C
-  bdg_status update_full(const T* bank, int P, const HostMat& C, T* Y, int Q) {
-    PairBlock<R> A{bank, vlen_, vlen_, P};
-    return update(A, C, 0.0, Y, Q);
   }
 
   // ---- start block --------------------------------------------------------
