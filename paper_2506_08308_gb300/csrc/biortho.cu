@@ -76,72 +76,60 @@ __global__ void k_jw_embed(const double* __restrict__ G, int n, double* __restri
 // are not (numerically) in the span of the kept vectors and their J-images
 // -- a Gram-Schmidt against both, which also handles degenerate clusters
 // where the eigensolver returns an arbitrary real basis of the eigenspace.
-// One CTA; out: E (M x M row-major, kept vectors in columns 0..), wsel, *count.
+// One CTA of a thread per component, which keeps the candidate; out: E (M x M
+// row-major, kept vectors in columns 0..), wsel, *count.  A serial chain: per
+// candidate, kept vector and pass one reduction over the CTA, with one barrier
+// (every warp adds the warps' sums itself, in their order) and the kept
+// vectors in shared memory.
 __global__ void k_jw_select(const double* __restrict__ V, const double* __restrict__ w, int M, int c_lo,
                             int max_keep, double* __restrict__ E, double* __restrict__ wsel, int* count) {
-  extern __shared__ double sh[];
-  double* e = sh;            // [M]
-  double* red = sh + M;      // [32]
-  const int tid = threadIdx.x, h = M / 2;
-  int kept = 0;
+  extern __shared__ double Es[];   // [max_keep][M]
+  __shared__ double red[2][2][8];
+  const int i = threadIdx.x, h = M / 2, warp = i >> 5, nw = blockDim.x / 32;
+  const bool on = i < M;
+  int kept = 0, buf = 0;
+  double nextv = on ? V[(long long)i * M + M - 1] : 0.0;
   for (int c = M - 1; c >= c_lo && kept < max_keep; --c) {
-    for (int i = tid; i < M; i += blockDim.x) e[i] = V[(long long)i * M + c];
-    __syncthreads();
+    double e = nextv;
+    if (on && c > c_lo) nextv = V[(long long)i * M + c - 1];
     for (int pass = 0; pass < 2; ++pass) {
-      for (int j = 0; j < kept; ++j) {
+      for (int j = 0; j < kept; ++j, buf ^= 1) {
         // d1 = E_j . e, d2 = (J E_j) . e with J E_j = [-E_j(h:); E_j(:h)]
-        double d1 = 0.0, d2 = 0.0;
-        for (int i = tid; i < M; i += blockDim.x) {
-          const double ej = E[(long long)i * M + j];
-          const double jej = i < h ? -E[(long long)(i + h) * M + j] : E[(long long)(i - h) * M + j];
-          d1 += ej * e[i];
-          d2 += jej * e[i];
+        const double* Ej = Es + j * M;
+        double ej = 0.0, jej = 0.0;
+        if (on) {
+          ej = Ej[i];
+          jej = i < h ? -Ej[i + h] : Ej[i - h];
         }
+        double d1 = ej * e, d2 = jej * e;
         for (int o = 16; o > 0; o >>= 1) {
           d1 += __shfl_xor_sync(0xffffffffu, d1, o);
           d2 += __shfl_xor_sync(0xffffffffu, d2, o);
         }
-        if ((tid & 31) == 0) { red[tid >> 5] = d1; red[16 + (tid >> 5)] = d2; }
+        if ((i & 31) == 0) { red[buf][0][warp] = d1; red[buf][1][warp] = d2; }
         __syncthreads();
-        if (tid == 0) {
-          double a = 0.0, b = 0.0;
-          for (int q = 0; q < (int)blockDim.x / 32; ++q) { a += red[q]; b += red[16 + q]; }
-          red[0] = a;
-          red[16] = b;
-        }
-        __syncthreads();
-        d1 = red[0];
-        d2 = red[16];
-        __syncthreads();
-        for (int i = tid; i < M; i += blockDim.x) {
-          const double ej = E[(long long)i * M + j];
-          const double jej = i < h ? -E[(long long)(i + h) * M + j] : E[(long long)(i - h) * M + j];
-          e[i] -= d1 * ej + d2 * jej;
-        }
-        __syncthreads();
+        d1 = red[buf][0][0];
+        d2 = red[buf][1][0];
+        for (int q = 1; q < nw; ++q) { d1 += red[buf][0][q]; d2 += red[buf][1][q]; }
+        e -= d1 * ej + d2 * jej;
       }
     }
-    double nn = 0.0;
-    for (int i = tid; i < M; i += blockDim.x) nn += e[i] * e[i];
+    double nn = e * e;
     for (int o = 16; o > 0; o >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, o);
-    if ((tid & 31) == 0) red[tid >> 5] = nn;
+    if ((i & 31) == 0) red[buf][0][warp] = nn;
     __syncthreads();
-    if (tid == 0) {
-      double a = 0.0;
-      for (int q = 0; q < (int)blockDim.x / 32; ++q) a += red[q];
-      red[0] = a;
-    }
-    __syncthreads();
-    const double nrm = sqrt(red[0]);
-    __syncthreads();
+    nn = red[buf][0][0];
+    for (int q = 1; q < nw; ++q) nn += red[buf][0][q];
+    buf ^= 1;
+    const double nrm = sqrt(nn);
     if (nrm > 0.5) {   // a unit candidate mostly outside the kept span
-      for (int i = tid; i < M; i += blockDim.x) E[(long long)i * M + kept] = e[i] / nrm;
-      if (tid == 0) wsel[kept] = w[c];
+      if (on) E[(long long)i * M + kept] = Es[kept * M + i] = e / nrm;
+      if (i == 0) wsel[kept] = w[c];
       ++kept;
+      __syncthreads();
     }
-    __syncthreads();
   }
-  if (tid == 0) *count = kept;
+  if (i == 0) *count = kept;
 }
 
 // From the selected eigenvectors e_k = [a; b] of R (4n x 4n, columns idx[k]):
@@ -232,7 +220,9 @@ struct Bio {
     double* E = sc + 256;                      // M x M (kept vectors in its first columns)
     double* wsel = E + 160 * 160;
     int* dcount = (int*)(wsel + 128);
-    k_jw_select<<<1, 256, sizeof(double) * (M + 32), s>>>(Vm, w, M, c_lo, ncol, E, wsel, dcount);
+    const size_t smsel = sizeof(double) * (size_t)ncol * M;
+    BDG_CUDA_TRY(plan, allow_dynamic_smem((const void*)k_jw_select, smsel));
+    k_jw_select<<<1, (M + 31) / 32 * 32, smsel, s>>>(Vm, w, M, c_lo, ncol, E, wsel, dcount);
     BDG_CUDA_TRY(plan, cudaGetLastError());
     int r = 0;
     std::vector<double> hsel(ncol);

@@ -46,133 +46,6 @@ __global__ void k_dgemm(bool ta, bool tb, int m, int n, int k, double alpha, con
   }
 }
 
-// ---------------------------------------------------------------------------
-// Parallel cyclic Jacobi (FP32) on one CTA: round-robin ordering, each round
-// rotates n/2 disjoint (p, q) planes, rows then columns.  Rotation of
-// Golub & Van Loan (sym.schur2): tau = (a_qq - a_pp) / (2 a_pq),
-// t = sign(tau) / (|tau| + sqrt(1 + tau^2)), c = 1/sqrt(1+t^2), s = t c.
-// Output ascending eigenvalues and the matching columns of V (FP64 copies).
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_jacobi(int n, const double* __restrict__ Ag, int lda,
-                                                 double* __restrict__ w, double* __restrict__ Vg,
-                                                 int max_sweeps, float off_tol) {
-  extern __shared__ float sm[];
-  const int ld = n + 1;
-  float* A = sm;                 // [n][ld]
-  float* V = A + n * ld;         // [n][ld]
-  float* cs = V + n * ld;        // [npair][2]
-  int* pq = (int*)(cs + 2 * (n / 2 + 1));  // [npair][2]
-  float* red = (float*)(pq + 2 * (n / 2 + 1));  // [64]
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int np2 = (n + 1) & ~1;  // even count including a dummy index
-  const int npair = np2 / 2;
-  for (int e = tid; e < n * n; e += nt) {
-    const int i = e / n, j = e - i * n;
-    A[i * ld + j] = (float)Ag[(long long)i * lda + j];
-    V[i * ld + j] = (i == j) ? 1.f : 0.f;
-  }
-  __syncthreads();
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    // off-diagonal and total Frobenius norms
-    float off = 0.f, tot = 0.f;
-    for (int e = tid; e < n * n; e += nt) {
-      const int i = e / n, j = e - i * n;
-      const float v = A[i * ld + j];
-      tot += v * v;
-      if (i != j) off += v * v;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      off += __shfl_xor_sync(0xffffffffu, off, o);
-      tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    }
-    if ((tid & 31) == 0) { red[tid >> 5] = off; red[32 + (tid >> 5)] = tot; }
-    __syncthreads();
-    if (tid == 0) {
-      float so = 0.f, st = 0.f;
-      for (int q = 0; q < (nt + 31) / 32; ++q) { so += red[q]; st += red[32 + q]; }
-      red[0] = so;
-      red[32] = st;
-    }
-    __syncthreads();
-    const bool done = red[0] <= off_tol * red[32];
-    __syncthreads();
-    if (done) break;
-    for (int r = 0; r < np2 - 1; ++r) {
-      if (tid < npair) {
-        const int k = tid;
-        int p = (r + k) % (np2 - 1);
-        int q = (k == 0) ? (np2 - 1) : (r - k + np2 - 1) % (np2 - 1);
-        if (p > q) { const int t = p; p = q; q = t; }
-        float c = 1.f, s = 0.f;
-        if (q < n) {
-          const float apq = A[p * ld + q];
-          const float app = A[p * ld + p], aqq = A[q * ld + q];
-          if (fabsf(apq) > 1e-30f && fabsf(apq) > 1e-9f * sqrtf(fabsf(app * aqq))) {
-            const float tau = (aqq - app) / (2.f * apq);
-            const float t = (tau >= 0.f ? 1.f : -1.f) / (fabsf(tau) + sqrtf(1.f + tau * tau));
-            c = rsqrtf(1.f + t * t);
-            s = t * c;
-          }
-        } else {
-          q = p;  // dummy: no rotation
-        }
-        pq[2 * k] = p;
-        pq[2 * k + 1] = q;
-        cs[2 * k] = c;
-        cs[2 * k + 1] = s;
-      }
-      __syncthreads();
-      // A <- J^T A J and V <- V J in one pass: a work item is the 2 x 2 block
-      // (row pair k, column pair l) of A -- rows first, then columns, as the
-      // two one-sided updates would do -- or the rows of V's column pair l.
-      // Warps take row pairs (or V's column pairs), lanes column pairs (or
-      // rows): no index division, and the row pair's indices and rotation
-      // are broadcast loads.  A dummy pair (odd n) has p == q and c = 1,
-      // s = 0, which makes its duplicate reads and writes agree.
-      const int lane = tid & 31, warp = tid >> 5, nwarp = nt >> 5;
-      for (int k = warp; k < npair; k += nwarp) {
-        const int p = pq[2 * k], q = pq[2 * k + 1];
-        const float ck = cs[2 * k], sk = cs[2 * k + 1];
-        float* Ap = A + p * ld;
-        float* Aq = A + q * ld;
-        for (int l = lane; l < npair; l += 32) {
-          const int u = pq[2 * l], v = pq[2 * l + 1];
-          const float cl = cs[2 * l], sl = cs[2 * l + 1];
-          const float x00 = Ap[u], x01 = Ap[v], x10 = Aq[u], x11 = Aq[v];
-          const float r00 = ck * x00 - sk * x10, r01 = ck * x01 - sk * x11;
-          const float r10 = sk * x00 + ck * x10, r11 = sk * x01 + ck * x11;
-          Ap[u] = cl * r00 - sl * r01;
-          Ap[v] = sl * r00 + cl * r01;
-          Aq[u] = cl * r10 - sl * r11;
-          Aq[v] = sl * r10 + cl * r11;
-        }
-      }
-      for (int l = warp; l < npair; l += nwarp) {
-        const int u = pq[2 * l], v = pq[2 * l + 1];
-        if (u == v) continue;
-        const float cl = cs[2 * l], sl = cs[2 * l + 1];
-        for (int i = lane; i < n; i += 32) {
-          const float vp = V[i * ld + u], vq = V[i * ld + v];
-          V[i * ld + u] = cl * vp - sl * vq;
-          V[i * ld + v] = sl * vp + cl * vq;
-        }
-      }
-      __syncthreads();
-    }
-  }
-  // ascending order by rank of the diagonal
-  for (int j = tid; j < n; j += nt) {
-    const float dj = A[j * ld + j];
-    int rank = 0;
-    for (int l = 0; l < n; ++l) {
-      const float dl = A[l * ld + l];
-      rank += (dl < dj) || (dl == dj && l < j);
-    }
-    w[rank] = (double)dj;
-    for (int i = 0; i < n; ++i) Vg[(long long)i * n + rank] = (double)V[i * ld + j];
-  }
-}
-
 // One Ogita-Aishima correction (SIAM J. Sci. Comput. 2018), given R = X^T X
 // and S = X^T A X: lam_i = s_ii / (1 - r_ii), with r = I - X^T X;
 // E_ij = (s_ij + lam_j r_ij) / (lam_j - lam_i) for pairs the current X
@@ -336,7 +209,7 @@ namespace {
 // shift c: two FP64 Newton-Schulz steps orthonormalize the columns, the
 // shifted projection G = Vs^T (A - c I) Vs (norm about half the run's
 // spread) is diagonalized by parallel cyclic Jacobi in FP64 (rotations of
-// Golub & Van Loan, round-robin pairs as in k_jacobi), and the rotated
+// Golub & Van Loan, round-robin pairs as in jacobi.cu), and the rotated
 // columns and eigenvalues (ascending within the run) replace the old ones.
 // ---------------------------------------------------------------------------
 constexpr int RC_MAX_CLUSTERS = 96;   // runs of two or more columns: at most n / 2
@@ -350,8 +223,8 @@ struct ClusterList {
 
 size_t resolve_smem_bytes(int n, int ns) {
   const int np2 = (ns + 1) & ~1;
-  return sizeof(double) * (2 * (size_t)n * ns + 2 * (size_t)ns * ns + 2 * (size_t)np2 + 64) +
-         sizeof(int) * ((size_t)np2 + 2 * (size_t)ns + 8);
+  return sizeof(double) * (2 * (size_t)n * ns + 2 * (size_t)ns * (ns | 1) + 4 * (size_t)np2 + 64) +
+         sizeof(int) * (2 * (size_t)np2 + 2 * (size_t)ns + 8);
 }
 
 __global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* __restrict__ A, int lda,
@@ -363,12 +236,13 @@ __global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* _
   const int np2 = (ns + 1) & ~1, npair = np2 / 2;
   double* Vs = rsm;                       // [n][ns]
   double* T = Vs + (size_t)n * ns;        // [n][ns]
-  double* G = T + (size_t)n * ns;         // [ns][ns]
-  double* Z = G + (size_t)ns * ns;        // [ns][ns]
-  double* cs = Z + (size_t)ns * ns;       // [npair][2]
-  double* red = cs + np2;                 // [64]
-  int* pq = reinterpret_cast<int*>(red + 64);   // [npair][2]
-  int* rank = pq + np2;                   // [ns]
+  const int ld = ns | 1;                  // odd: Z is rotated down its columns
+  double* G = T + (size_t)n * ns;         // [ns][ld]
+  double* Z = G + (size_t)ns * ld;        // [ns][ld]
+  double* cs = Z + (size_t)ns * ld;       // [2][npair][2]: this round's rotations and the next's
+  double* red = cs + 2 * np2;             // [64]
+  int* pq = reinterpret_cast<int*>(red + 64);   // [2][npair][2]
+  int* rank = pq + 2 * np2;               // [ns]
   const int tid = threadIdx.x, nt = blockDim.x;
   for (int e = tid; e < n * ns; e += nt) {
     const int i = e / ns, j = e - i * ns;
@@ -381,13 +255,13 @@ __global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* _
       const int a = e / ns, b = e - a * ns;
       double sacc = 0.0;
       for (int i = 0; i < n; ++i) sacc = fma(Vs[i * ns + a], Vs[i * ns + b], sacc);
-      G[e] = (a == b ? 1.5 : 0.0) - 0.5 * sacc;
+      G[a * ld + b] = (a == b ? 1.5 : 0.0) - 0.5 * sacc;
     }
     __syncthreads();
     for (int e = tid; e < n * ns; e += nt) {
       const int i = e / ns, b = e - i * ns;
       double sacc = 0.0;
-      for (int a = 0; a < ns; ++a) sacc = fma(Vs[i * ns + a], G[a * ns + b], sacc);
+      for (int a = 0; a < ns; ++a) sacc = fma(Vs[i * ns + a], G[a * ld + b], sacc);
       T[e] = sacc;
     }
     __syncthreads();
@@ -407,14 +281,14 @@ __global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* _
     const int a = e / ns, b = e - a * ns;
     double sacc = 0.0;
     for (int i = 0; i < n; ++i) sacc = fma(Vs[i * ns + a], T[i * ns + b], sacc);
-    Z[e] = sacc;
+    Z[a * ld + b] = sacc;
   }
   __syncthreads();
   double fro = 0.0;
   for (int e = tid; e < ns * ns; e += nt) {
     const int a = e / ns, b = e - a * ns;
-    const double v = 0.5 * (Z[a * ns + b] + Z[b * ns + a]);
-    G[e] = v;
+    const double v = 0.5 * (Z[a * ld + b] + Z[b * ld + a]);
+    G[a * ld + b] = v;
     fro += v * v;
   }
   for (int o = 16; o > 0; o >>= 1) fro += __shfl_xor_sync(0xffffffffu, fro, o);
@@ -425,7 +299,7 @@ __global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* _
     for (int q = 0; q < (nt + 31) / 32; ++q) t += red[q];
     red[32] = sqrt(t);
   }
-  for (int e = tid; e < ns * ns; e += nt) Z[e] = (e / ns == e % ns) ? 1.0 : 0.0;
+  for (int e = tid; e < ns * ns; e += nt) Z[e / ns * ld + e % ns] = (e / ns == e % ns) ? 1.0 : 0.0;
   __syncthreads();
   const double tiny = 1e-18 * red[32];
   // parallel cyclic Jacobi in FP64
@@ -433,7 +307,8 @@ __global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* _
     double off = 0.0;
     for (int e = tid; e < ns * ns; e += nt) {
       const int a = e / ns, b = e - a * ns;
-      if (a != b) off += G[e] * G[e];
+      const double v = G[a * ld + b];
+      if (a != b) off += v * v;
     }
     for (int o = 16; o > 0; o >>= 1) off += __shfl_xor_sync(0xffffffffu, off, o);
     __syncthreads();
@@ -446,7 +321,10 @@ __global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* _
     }
     __syncthreads();
     if (!(red[33] > 1e-32 * red[32] * red[32]) || !(red[33] > tiny * tiny)) break;
-    for (int r = 0; r < np2 - 1; ++r) {
+    // The rotations of round r + 1 need the matrix of round r, but not Z: the
+    // first warp forms them (a chain of divisions and square roots) while the
+    // others rotate Z.  Per round the FP64 pipe of the SM bounds both parts.
+    auto rotations = [&](int r, int set) {
       if (tid < npair) {
         const int k = tid;
         int p = (r + k) % (np2 - 1);
@@ -454,7 +332,7 @@ __global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* _
         if (p > q) { const int t = p; p = q; q = t; }
         double cc = 1.0, ss = 0.0;
         if (q < ns) {
-          const double apq = G[p * ns + q], app = G[p * ns + p], aqq = G[q * ns + q];
+          const double apq = G[p * ld + q], app = G[p * ld + p], aqq = G[q * ld + q];
           if (fabs(apq) > tiny) {
             const double tau = (aqq - app) / (2.0 * apq);
             const double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
@@ -464,44 +342,52 @@ __global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* _
         } else {
           q = p;
         }
-        pq[2 * k] = p;
-        pq[2 * k + 1] = q;
-        cs[2 * k] = cc;
-        cs[2 * k + 1] = ss;
+        pq[set * np2 + 2 * k] = p;
+        pq[set * np2 + 2 * k + 1] = q;
+        cs[set * np2 + 2 * k] = cc;
+        cs[set * np2 + 2 * k + 1] = ss;
+      }
+    };
+    rotations(0, 0);
+    for (int r = 0; r < np2 - 1; ++r) {
+      const int* pqr = pq + (r & 1) * np2;
+      const double* csr = cs + (r & 1) * np2;
+      __syncthreads();
+      for (int e = tid; e < npair * npair; e += nt) {
+        const int k = e / npair, l = e - k * npair;
+        const int p = pqr[2 * k], q = pqr[2 * k + 1], u = pqr[2 * l], v = pqr[2 * l + 1];
+        const double ck = csr[2 * k], sk = csr[2 * k + 1], cl_ = csr[2 * l], sl = csr[2 * l + 1];
+        const double x00 = G[p * ld + u], x01 = G[p * ld + v], x10 = G[q * ld + u], x11 = G[q * ld + v];
+        const double r00 = ck * x00 - sk * x10, r01 = ck * x01 - sk * x11;
+        const double r10 = sk * x00 + ck * x10, r11 = sk * x01 + ck * x11;
+        G[p * ld + u] = cl_ * r00 - sl * r01;
+        G[p * ld + v] = sl * r00 + cl_ * r01;
+        G[q * ld + u] = cl_ * r10 - sl * r11;
+        G[q * ld + v] = sl * r10 + cl_ * r11;
       }
       __syncthreads();
-      const int nblk = npair * npair;
-      for (int e = tid; e < nblk + npair * ns; e += nt) {
-        if (e < nblk) {
-          const int k = e / npair, l = e - k * npair;
-          const int p = pq[2 * k], q = pq[2 * k + 1], u = pq[2 * l], v = pq[2 * l + 1];
-          const double ck = cs[2 * k], sk = cs[2 * k + 1], cl_ = cs[2 * l], sl = cs[2 * l + 1];
-          const double x00 = G[p * ns + u], x01 = G[p * ns + v], x10 = G[q * ns + u], x11 = G[q * ns + v];
-          const double r00 = ck * x00 - sk * x10, r01 = ck * x01 - sk * x11;
-          const double r10 = sk * x00 + ck * x10, r11 = sk * x01 + ck * x11;
-          G[p * ns + u] = cl_ * r00 - sl * r01;
-          G[p * ns + v] = sl * r00 + cl_ * r01;
-          G[q * ns + u] = cl_ * r10 - sl * r11;
-          G[q * ns + v] = sl * r10 + cl_ * r11;
-        } else {
-          const int f = e - nblk, l = f / ns, i = f - l * ns;
-          const int u = pq[2 * l], v = pq[2 * l + 1];
+      if (tid < 32) {   // (npair <= 24 lanes of one warp)
+        if (r + 1 < np2 - 1) rotations(r + 1, (r + 1) & 1);
+      } else {
+        for (int f = tid - 32; f < npair * ns; f += nt - 32) {
+          const int l = f / ns, i = f - l * ns;
+          const int u = pqr[2 * l], v = pqr[2 * l + 1];
           if (u == v) continue;
-          const double cl_ = cs[2 * l], sl = cs[2 * l + 1];
-          const double zp = Z[i * ns + u], zq = Z[i * ns + v];
-          Z[i * ns + u] = cl_ * zp - sl * zq;
-          Z[i * ns + v] = sl * zp + cl_ * zq;
+          const double cl_ = csr[2 * l], sl = csr[2 * l + 1];
+          const double zp = Z[i * ld + u], zq = Z[i * ld + v];
+          Z[i * ld + u] = cl_ * zp - sl * zq;
+          Z[i * ld + v] = sl * zp + cl_ * zq;
         }
       }
-      __syncthreads();
     }
+    __syncthreads();
   }
   // ascending order within the run, new columns Vs Z, eigenvalues + c
   for (int j = tid; j < ns; j += nt) {
-    const double dj = G[j * ns + j];
+    const double dj = G[j * ld + j];
     int rk = 0;
     for (int l = 0; l < ns; ++l) {
-      const double dl = G[l * ns + l];
+      const double dl = G[l * ld + l];
       rk += (dl < dj) || (dl == dj && l < j);
     }
     rank[j] = rk;
@@ -511,7 +397,7 @@ __global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* _
   for (int e = tid; e < n * ns; e += nt) {
     const int i = e / ns, j = e - i * ns;
     double sacc = 0.0;
-    for (int a = 0; a < ns; ++a) sacc = fma(Vs[i * ns + a], Z[a * ns + j], sacc);
+    for (int a = 0; a < ns; ++a) sacc = fma(Vs[i * ns + a], Z[a * ld + j], sacc);
     V[(long long)i * n + i0 + rank[j]] = sacc;
   }
 }
@@ -525,10 +411,7 @@ __global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* _
 // the workspace is reused from one to the next.
 cudaError_t jacobi_multilevel(int n, const double* A, int lda, double* w, double* V, double* ws, int depth,
                               double floor, double shift, cudaStream_t s) {
-  const size_t sm = sizeof(float) * (2 * (size_t)n * (n + 1) + 2 * (n / 2 + 1)) +
-                    sizeof(int) * 2 * (n / 2 + 1) + sizeof(float) * 64;
-  cudaError_t e = allow_dynamic_smem((const void*)k_jacobi, sm);
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
   static const bool prof = getenv("BDG_PROFILE_EIGH") != nullptr;
   cudaEvent_t pj[2] = {};
   if (prof) {
@@ -536,10 +419,7 @@ cudaError_t jacobi_multilevel(int n, const double* A, int lda, double* w, double
     cudaEventCreate(&pj[1]);
     cudaEventRecord(pj[0], s);
   }
-  // converged to off(A) <= 1e-12 |A|^2: the FP64 refinement needs a start
-  // this close (a stop at 1e-7 left backward errors up to 5e-2)
-  k_jacobi<<<1, 1024, sm, s>>>(n, A, lda, w, V, 30, 1e-12f);
-  if ((e = cudaGetLastError())) return e;
+  if ((e = jacobi_f32(n, A, lda, w, V, s))) return e;
   if (prof) {
     cudaEventRecord(pj[1], s);
     cudaEventSynchronize(pj[1]);

@@ -14,7 +14,7 @@ cudaError_t dgemm_small(bool ta, bool tb, int m, int n, int k, double alpha, con
                         const double* B, int ldb, double beta, double* C, int ldc, cudaStream_t s);
 
 // Symmetric eigen-decomposition A = V diag(w) V^T of an n x n FP64 matrix
-// (row-major, lda), ascending w.  Parallel cyclic Jacobi in FP32 on one CTA
+// (row-major, lda), ascending w.  Parallel cyclic Jacobi in FP32 (jacobi.cu)
 // gives a first V; Ogita-Aishima refinement steps in FP64 (SIAM J. Sci.
 // Comput. 2018 "Iterative refinement for symmetric eigenvalue
 // decomposition") bring it to FP64 accuracy.  ws: workspace of
@@ -28,6 +28,10 @@ size_t eigh_workspace_doubles(int n);
 // hundred times its coupling).
 cudaError_t eigh(int n, const double* A, int lda, double* w, double* V, double* ws, int refine_steps,
                  cudaStream_t s, double floor_rel = 0.0, bool from_identity = false);
+
+// Its first stage: eigenvalues (ascending) and eigenvectors (columns of V, ld
+// n) of A rounded to FP32, by cyclic Jacobi to off(A)^2 <= 1e-12 |A|^2.
+cudaError_t jacobi_f32(int n, const double* A, int lda, double* w, double* V, cudaStream_t s);
 
 // Rank-revealing Cholesky factorization with symmetric pivoting of a
 // symmetric positive semidefinite n x n FP64 matrix A (row-major, lda):
