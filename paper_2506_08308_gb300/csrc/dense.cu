@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "dense.cuh"
+#include "jacobi.cuh"
 
 namespace bdg {
 
@@ -221,29 +222,35 @@ struct ClusterList {
   double shift[RC_MAX_CLUSTERS];
 };
 
-size_t resolve_smem_bytes(int n, int ns) {
-  const int np2 = (ns + 1) & ~1;
-  return sizeof(double) * (2 * (size_t)n * ns + 2 * (size_t)ns * (ns | 1) + 4 * (size_t)np2 + 64) +
-         sizeof(int) * (2 * (size_t)np2 + 2 * (size_t)ns + 8);
-}
+// The rotation that annihilates apq (above the rounding level tiny).  For
+// |tau| > 2^28, sqrt(1 + tau^2) rounds to |tau| and 1 + t^2 to 1: the short
+// form gives the same bits without two square roots and a division.
+struct Rotation64 {
+  double tiny;
+  __device__ __forceinline__ void operator()(double app, double apq, double aqq, double& c, double& s) const {
+    c = 1.0;
+    s = 0.0;
+    if (fabs(apq) > tiny) {
+      const double tau = (aqq - app) / (2.0 * apq), at = fabs(tau), sg = tau >= 0.0 ? 1.0 : -1.0;
+      if (at > 0x1p28 && at < 0x1p500) {
+        s = sg / (at + at);
+      } else {
+        const double t = sg / (at + sqrt(1.0 + tau * tau));
+        c = 1.0 / sqrt(1.0 + t * t);
+        s = t * c;
+      }
+    }
+  }
+};
 
-__global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* __restrict__ A, int lda,
-                                                          double* __restrict__ w, double* __restrict__ V,
-                                                          ClusterList cl) {
-  extern __shared__ double rsm[];
-  const int i0 = cl.start[blockIdx.x], ns = cl.size[blockIdx.x];
-  const double c = cl.shift[blockIdx.x];
-  const int np2 = (ns + 1) & ~1, npair = np2 / 2;
-  double* Vs = rsm;                       // [n][ns]
-  double* T = Vs + (size_t)n * ns;        // [n][ns]
-  const int ld = ns | 1;                  // odd: Z is rotated down its columns
-  double* G = T + (size_t)n * ns;         // [ns][ld]
-  double* Z = G + (size_t)ns * ld;        // [ns][ld]
-  double* cs = Z + (size_t)ns * ld;       // [2][npair][2]: this round's rotations and the next's
-  double* red = cs + 2 * np2;             // [64]
-  int* pq = reinterpret_cast<int*>(red + 64);   // [2][npair][2]
-  int* rank = pq + 2 * np2;               // [ns]
-  const int tid = threadIdx.x, nt = blockDim.x;
+constexpr int RT = 256;   // threads of a CTA of the resolving kernels
+
+// What both resolving kernels begin with, on one CTA: the run's columns of V
+// orthonormalized in Vs, their shifted projection in G ([ns][ld]) and, for
+// every thread, its Frobenius norm.  T: n x ns, Z: like G, red: 34 values.
+__device__ double resolve_project(int n, const double* __restrict__ A, int lda, const double* V, int i0, int ns,
+                                  double c, int ld, double* Vs, double* T, double* G, double* Z, double* red) {
+  const int tid = threadIdx.x, nt = RT;
   for (int e = tid; e < n * ns; e += nt) {
     const int i = e / ns, j = e - i * ns;
     Vs[e] = V[(long long)i * n + i0 + j];
@@ -296,12 +303,41 @@ __global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* _
   __syncthreads();
   if (tid == 0) {
     double t = 0.0;
-    for (int q = 0; q < (nt + 31) / 32; ++q) t += red[q];
+    for (int q = 0; q < nt / 32; ++q) t += red[q];
     red[32] = sqrt(t);
   }
+  __syncthreads();
+  return red[32];
+}
+
+size_t resolve_smem_bytes(int n, int ns) {
+  const int np2 = (ns + 1) & ~1;
+  return sizeof(double) * (2 * (size_t)n * ns + 2 * (size_t)ns * (ns | 1) + 4 * (size_t)np2 + 64) +
+         sizeof(int) * (2 * (size_t)np2 + 2 * (size_t)ns + 8);
+}
+
+__global__ void __launch_bounds__(RT) k_resolve_clusters(int n, const double* __restrict__ A, int lda,
+                                                         double* __restrict__ w, double* __restrict__ V,
+                                                         ClusterList cl) {
+  extern __shared__ double rsm[];
+  const int i0 = cl.start[blockIdx.x], ns = cl.size[blockIdx.x];
+  const double c = cl.shift[blockIdx.x];
+  const int np2 = (ns + 1) & ~1, npair = np2 / 2;
+  double* Vs = rsm;                       // [n][ns]
+  double* T = Vs + (size_t)n * ns;        // [n][ns]
+  const int ld = ns | 1;                  // odd: Z is rotated down its columns
+  double* G = T + (size_t)n * ns;         // [ns][ld]
+  double* Z = G + (size_t)ns * ld;        // [ns][ld]
+  double* cs = Z + (size_t)ns * ld;       // [2][npair][2]: this round's rotations and the next's
+  double* red = cs + 2 * np2;             // [64]
+  int* pq = reinterpret_cast<int*>(red + 64);   // [2][npair][2]
+  int* rank = pq + 2 * np2;               // [ns]
+  const int tid = threadIdx.x, nt = RT;
+  const double fro = resolve_project(n, A, lda, V, i0, ns, c, ld, Vs, T, G, Z, red);
   for (int e = tid; e < ns * ns; e += nt) Z[e / ns * ld + e % ns] = (e / ns == e % ns) ? 1.0 : 0.0;
   __syncthreads();
-  const double tiny = 1e-18 * red[32];
+  const double tiny = 1e-18 * fro;
+  const Rotation64 rotate{tiny};
   // parallel cyclic Jacobi in FP64
   for (int sweep = 0; sweep < 40; ++sweep) {
     double off = 0.0;
@@ -320,7 +356,7 @@ __global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* _
       red[33] = t;
     }
     __syncthreads();
-    if (!(red[33] > 1e-32 * red[32] * red[32]) || !(red[33] > tiny * tiny)) break;
+    if (!(red[33] > 1e-32 * fro * fro) || !(red[33] > tiny * tiny)) break;
     // The rotations of round r + 1 need the matrix of round r, but not Z: the
     // first warp forms them (a chain of divisions and square roots) while the
     // others rotate Z.  Per round the FP64 pipe of the SM bounds both parts.
@@ -332,13 +368,7 @@ __global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* _
         if (p > q) { const int t = p; p = q; q = t; }
         double cc = 1.0, ss = 0.0;
         if (q < ns) {
-          const double apq = G[p * ld + q], app = G[p * ld + p], aqq = G[q * ld + q];
-          if (fabs(apq) > tiny) {
-            const double tau = (aqq - app) / (2.0 * apq);
-            const double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-            cc = 1.0 / sqrt(1.0 + t * t);
-            ss = t * cc;
-          }
+          rotate(G[p * ld + p], G[p * ld + q], G[q * ld + q], cc, ss);
         } else {
           q = p;
         }
@@ -356,14 +386,12 @@ __global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* _
       for (int e = tid; e < npair * npair; e += nt) {
         const int k = e / npair, l = e - k * npair;
         const int p = pqr[2 * k], q = pqr[2 * k + 1], u = pqr[2 * l], v = pqr[2 * l + 1];
-        const double ck = csr[2 * k], sk = csr[2 * k + 1], cl_ = csr[2 * l], sl = csr[2 * l + 1];
-        const double x00 = G[p * ld + u], x01 = G[p * ld + v], x10 = G[q * ld + u], x11 = G[q * ld + v];
-        const double r00 = ck * x00 - sk * x10, r01 = ck * x01 - sk * x11;
-        const double r10 = sk * x00 + ck * x10, r11 = sk * x01 + ck * x11;
-        G[p * ld + u] = cl_ * r00 - sl * r01;
-        G[p * ld + v] = sl * r00 + cl_ * r01;
-        G[q * ld + u] = cl_ * r10 - sl * r11;
-        G[q * ld + v] = sl * r10 + cl_ * r11;
+        Block2<double> x{G[p * ld + u], G[p * ld + v], G[q * ld + u], G[q * ld + v]};
+        x.rotate(csr[2 * k], csr[2 * k + 1], csr[2 * l], csr[2 * l + 1]);
+        G[p * ld + u] = x.x00;
+        G[p * ld + v] = x.x01;
+        G[q * ld + u] = x.x10;
+        G[q * ld + v] = x.x11;
       }
       __syncthreads();
       if (tid < 32) {   // (npair <= 24 lanes of one warp)
@@ -375,8 +403,8 @@ __global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* _
           if (u == v) continue;
           const double cl_ = csr[2 * l], sl = csr[2 * l + 1];
           const double zp = Z[i * ld + u], zq = Z[i * ld + v];
-          Z[i * ld + u] = cl_ * zp - sl * zq;
-          Z[i * ld + v] = sl * zp + cl_ * zq;
+          Z[i * ld + u] = minus2(cl_, zp, sl, zq);
+          Z[i * ld + v] = plus2(sl, zp, cl_, zq);
         }
       }
     }
@@ -396,6 +424,78 @@ __global__ void __launch_bounds__(256) k_resolve_clusters(int n, const double* _
   __syncthreads();
   for (int e = tid; e < n * ns; e += nt) {
     const int i = e / ns, j = e - i * ns;
+    double sacc = 0.0;
+    for (int a = 0; a < ns; ++a) sacc = fma(Vs[i * ns + a], Z[a * ld + j], sacc);
+    V[(long long)i * n + i0 + rank[j]] = sacc;
+  }
+}
+
+// Wide runs on a cluster of eight CTAs (jacobi.cuh): the FP64 pipe of one SM
+// bounds a round there, and the many sweeps of a run that is degenerate to
+// working precision are serial.  Two runs of 48 such columns of n = 96: 9.9 ms
+// on one CTA each, 3.84 here; two of 42 (n = 128), resolved in a few sweeps:
+// whole eigensolve 9.8 -> 6.6 ms.  Narrower runs would leave a CTA of the
+// cluster without its two pair positions.
+constexpr int RC_WIDE = 32;
+typedef JShared<double, RC_NS_MAX, RT> RShared;
+
+size_t resolve_wide_smem_bytes(int n, int ns) {
+  return sizeof(RShared) + sizeof(double) * (2 * (size_t)n * ns + 2 * (size_t)ns * (ns | 1) + 64 + (size_t)RC_NS_MAX) +
+         sizeof(int) * (size_t)RC_NS_MAX;
+}
+
+__global__ void __cluster_dims__(JC, 1, 1) __launch_bounds__(RT)
+    k_resolve_wide(int n, const double* __restrict__ A, int lda, double* __restrict__ w, double* __restrict__ V,
+                   ClusterList cl) {
+  extern __shared__ double rsm[];
+  const int run = blockIdx.x / JC, cta = blockIdx.x % JC;
+  const int i0 = cl.start[run], ns = cl.size[run], ld = ns | 1;
+  const double c = cl.shift[run];
+  RShared& sh = *reinterpret_cast<RShared*>(rsm);
+  double* Vs = rsm + sizeof(RShared) / sizeof(double);   // [n][ns]
+  double* T = Vs + (size_t)n * ns;                       // [n][ns]
+  double* G = T + (size_t)n * ns;                        // [ns][ld]
+  double* Z = G + (size_t)ns * ld;                       // [ns][ld]
+  double* red = Z + (size_t)ns * ld;                     // [64]
+  double* diag = red + 64;                               // [RC_NS_MAX]
+  int* rank = reinterpret_cast<int*>(diag + RC_NS_MAX);  // [RC_NS_MAX]
+  const int tid = threadIdx.x;
+  const double fro = resolve_project(n, A, lda, V, i0, ns, c, ld, Vs, T, G, Z, red);   // (every CTA for itself)
+  const double tiny = 1e-18 * fro;
+  const int par = jacobi_sweeps(
+      sh, ns, cta, 40, [&](int i, int j) { return G[i * ld + j]; }, Rotation64{tiny},
+      [&](double off, double) { return !(off > 1e-32 * fro * fro) || !(off > tiny * tiny); });
+  // the rows of Z to every CTA
+  const int z0 = cta * ns / JC, zrows = (cta + 1) * ns / JC - z0;
+  __syncthreads();
+  for (int e = tid; e < zrows * ns; e += RT) {
+    const int i = e / ns, j = e - i * ns;
+    const uint32_t o = s_u32(Z + (z0 + i) * ld + j);
+    const double v = sh.V[i * RC_NS_MAX + j];
+    for (int d = 0; d < JC; ++d) put(at_cta(o, d), v);
+  }
+  // ascending order within the run, new columns Vs Z, eigenvalues + c
+  const int np2 = (ns + 1) & ~1;
+  if (tid < np2 / 2) {
+    diag[tid] = sh.next[par][0][tid];
+    if (np2 - 1 - tid < ns) diag[np2 - 1 - tid] = sh.next[par][2][tid];   // (round 0's pairs)
+  }
+  cluster_arrive();
+  cluster_wait();
+  for (int j = tid; j < ns; j += RT) {
+    const double dj = diag[j];
+    int rk = 0;
+    for (int l = 0; l < ns; ++l) {
+      const double dl = diag[l];
+      rk += (dl < dj) || (dl == dj && l < j);
+    }
+    rank[j] = rk;
+    if (cta == 0) w[i0 + rk] = dj + c;
+  }
+  __syncthreads();
+  const int r0 = cta * n / JC, r1 = (cta + 1) * n / JC;
+  for (int e = tid; e < (r1 - r0) * ns; e += RT) {
+    const int i = r0 + e / ns, j = e % ns;
     double sacc = 0.0;
     for (int a = 0; a < ns; ++a) sacc = fma(Vs[i * ns + a], Z[a * ld + j], sacc);
     V[(long long)i * n + i0 + rank[j]] = sacc;
@@ -440,9 +540,9 @@ cudaError_t jacobi_multilevel(int n, const double* A, int lda, double* w, double
   const double tau = 1e-4 * amax;
   // runs of at most RC_NS_MAX columns are resolved by one launch (FP64
   // Jacobi per run); wider runs re-solve in turn on their projection
-  ClusterList cl;
-  cl.count = 0;
-  int ns_max = 0;
+  ClusterList lists[2];   // narrow runs, wide ones
+  int ns_max[2] = {0, 0};
+  lists[0].count = lists[1].count = 0;
   for (int i0 = 0; i0 < n;) {
     int i1 = i0 + 1;
     while (i1 < n && hw[i1] - hw[i1 - 1] < tau) ++i1;
@@ -457,12 +557,13 @@ cudaError_t jacobi_multilevel(int n, const double* A, int lda, double* w, double
     // original matrix) are not needed resolved: the caller discards them
     const double top = std::max(std::fabs(hw[i0] + shift), std::fabs(hw[i1 - 1] + shift));
     if (ns >= 2 && spread > 0 && !degenerate && !(top < floor) && ns <= RC_NS_MAX &&
-        cl.count < RC_MAX_CLUSTERS) {
+        lists[ns >= RC_WIDE].count < RC_MAX_CLUSTERS) {
+      ClusterList& cl = lists[ns >= RC_WIDE];
       cl.start[cl.count] = i0;
       cl.size[cl.count] = ns;
       cl.shift[cl.count] = 0.5 * (hw[i0] + hw[i1 - 1]);
       cl.count++;
-      ns_max = std::max(ns_max, ns);
+      ns_max[ns >= RC_WIDE] = std::max(ns_max[ns >= RC_WIDE], ns);
     } else if (ns >= 2 && spread > 0 && !degenerate && !(top < floor)) {
       const double c = 0.5 * (hw[i0] + hw[i1 - 1]);  // midpoint: the shifted norm is half the spread
       double* Vs = ws;                         // n x ns
@@ -503,11 +604,18 @@ cudaError_t jacobi_multilevel(int n, const double* A, int lda, double* w, double
     i0 = i1;
   }
   if (prof && depth == 0)
-    fprintf(stderr, "[bdg]   clusters n %d: %d batched (widest %d)\n", n, cl.count, ns_max);
-  if (cl.count > 0) {
-    const size_t smr = resolve_smem_bytes(n, ns_max);
+    fprintf(stderr, "[bdg]   clusters n %d: %d batched (widest %d)\n", n, lists[0].count + lists[1].count,
+            std::max(ns_max[0], ns_max[1]));
+  if (lists[1].count > 0) {
+    const size_t smr = resolve_wide_smem_bytes(n, ns_max[1]);
+    if ((e = allow_dynamic_smem((const void*)k_resolve_wide, smr))) return e;
+    k_resolve_wide<<<JC * lists[1].count, RT, smr, s>>>(n, A, lda, w, V, lists[1]);
+    if ((e = cudaGetLastError())) return e;
+  }
+  if (lists[0].count > 0) {
+    const size_t smr = resolve_smem_bytes(n, ns_max[0]);
     if ((e = allow_dynamic_smem((const void*)k_resolve_clusters, smr))) return e;
-    k_resolve_clusters<<<cl.count, 256, smr, s>>>(n, A, lda, w, V, cl);
+    k_resolve_clusters<<<lists[0].count, RT, smr, s>>>(n, A, lda, w, V, lists[0]);
     if ((e = cudaGetLastError())) return e;
   }
   return cudaSuccess;
