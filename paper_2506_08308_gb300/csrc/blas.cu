@@ -375,9 +375,9 @@ size_t gram_workspace_bytes(int P, int Q, long long n) {
 bool gram_digits_pays(int P, int Q, long long n) { return P * Q > 1 && n >= 8192; }
 
 cudaError_t gram_pairs_fp64(const PairBlock<double>& A, const PairBlock<double>& B, double* G_dev, void* ws,
-                            size_t ws_bytes, cudaStream_t s, bool upper) {
+                            size_t ws_bytes, cudaStream_t s, bool upper, int digits) {
   if (A.n == B.n && gram_digits_pays(A.cols, B.cols, A.n) && gram_digits_fits(A.cols, B.cols, A.n, ws_bytes))
-    return gram_pairs_digits<double>(A, B, true, G_dev, ws, ws_bytes, s);
+    return gram_pairs_digits<double>(A, B, digits, G_dev, ws, ws_bytes, s);
   return gram_pairs<double>(A, B, G_dev, ws, ws_bytes, s, upper);
 }
 

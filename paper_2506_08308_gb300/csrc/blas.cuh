@@ -29,10 +29,11 @@ template <typename R>
 cudaError_t gram_pairs(const PairBlock<R>& A, const PairBlock<R>& B, double* G_dev, void* ws,
                        size_t ws_bytes, cudaStream_t s, bool upper = false);
 // FP64 Gram by digits where that pays (gram_digits_pays: long columns, more
-// than one pair), else by gram_pairs.
+// than one pair), else by gram_pairs.  digits: 6, or 7 where 2^-48 of a
+// column's largest value in 256 rows is too much.
 bool gram_digits_pays(int P, int Q, long long n);
 cudaError_t gram_pairs_fp64(const PairBlock<double>& A, const PairBlock<double>& B, double* G_dev, void* ws,
-                            size_t ws_bytes, cudaStream_t s, bool upper = false);
+                            size_t ws_bytes, cudaStream_t s, bool upper = false, int digits = 6);
 size_t gram_workspace_bytes(int P, int Q, long long n);
 
 // The same Gram (full, no triangle) on the tensor cores with split-BF16
@@ -44,13 +45,14 @@ cudaError_t gram_pairs_tc(const PairBlock<R>& A, const PairBlock<R>& B, double* 
                           size_t ws_bytes, cudaStream_t s);
 
 // The same Gram (full, no triangle) from exact integer digits on the tensor
-// cores (gram_digits.cu), with FP64 (FP64 blocks) or FP32 accuracy.  ws as for
+// cores (gram_digits.cu): 6 or 7 of them for FP64 accuracy (FP64 blocks), 4
+// for FP32 accuracy.  ws as for
 // gram_pairs; fewer row groups run in parallel if it is short, and
 // gram_digits_fits says whether it holds one.
 size_t gram_digits_workspace_bytes(int P, int Q, long long n);
 bool gram_digits_fits(int P, int Q, long long n, size_t ws_bytes);
 template <typename R>
-cudaError_t gram_pairs_digits(const PairBlock<R>& A, const PairBlock<R>& B, bool fp64, double* G_dev, void* ws,
+cudaError_t gram_pairs_digits(const PairBlock<R>& A, const PairBlock<R>& B, int digits, double* G_dev, void* ws,
                               size_t ws_bytes, cudaStream_t s);
 
 // Y[:, q].t = beta * Y[:, q].t + alpha * sum_{p,s} A[:, p].s * C[(2p+s) * ldc + 2q+t]

@@ -1,7 +1,7 @@
 // Tall-skinny Gram G = A^T B of two pair blocks on the tensor cores
 // (tcgen05.mma kind::f16, accumulators in tensor memory), from exact digits
 // (digits.cuh): FP64 accuracy with six digits per element (26 digit
-// products), FP32 accuracy with four (10 products).
+// products) or seven (34), FP32 accuracy with four (10).
 //
 // A CTA owns a tile of 128 x NT real columns and a range of row chunks of
 // CHUNK = 256 rows.  Every column has one exponent per chunk (k_col_exp),
@@ -22,7 +22,9 @@
 // 736 -> 138 us.  What bounds it now is the integer pipe of the producer
 // warps (52 % of its rate, 3300 clocks per 32-row stage against 2300 of the
 // MMAs, each of which reads 5.5 KB of operands at 128 bytes per clock); the
-// pass over the exponents takes 72 us at 80 % of the DRAM rate.
+// pass over the exponents takes 72 us at 80 % of the DRAM rate.  Seven digits
+// (the solver's projected problems) cost 24 x 24 pairs of 196608 rows 153 us for
+// the 133 of six, of the products alone.
 //
 // Operand tiles are MN-major without swizzle: a core matrix holds 8 rows (K)
 // of 8 neighbouring real columns (16 bytes), so that a thread that has one
@@ -39,14 +41,15 @@ namespace {
 
 constexpr int TM = 128;      // A real columns per CTA (MMA M)
 constexpr int TBK = 32;      // rows per pipeline stage (two MMA K steps of 16)
-constexpr int TSTAGES = 3;   // stages in flight
 constexpr int PWARPS = 16;   // warps that cut digits and read back; one more issues the MMAs
 constexpr int TTHREADS = 32 * (PWARPS + 1);
 constexpr int CHUNK = 256;   // rows per exponent and per read-back
 constexpr int STEPS = CHUNK / TBK;
 // digit weights kept: with six digits the seventh as well, whose five pairs
-// would otherwise be the largest error
-template <int ND> constexpr int weights() { return ND == 6 ? 7 : ND; }
+// would otherwise be the largest error, and with seven the eighth
+template <int ND> constexpr int weights() { return ND >= 6 ? ND + 1 : ND; }
+// stages in flight: what shared memory holds
+template <int ND> constexpr int stages() { return ND == 7 ? 2 : 3; }
 inline int padded8(int cols) { return (cols + 7) / 8 * 8; }
 
 // exps[chunk * ld + 2 c + part]: largest biased exponent of the column's real
@@ -143,7 +146,7 @@ template <typename R, int ND, int NT>
 __global__ void __launch_bounds__(TTHREADS, 1)
     k_gram_digits(PairBlock<R> A, PairBlock<R> B, const short* __restrict__ expA, const short* __restrict__ expB, int ldea,
               int ldeb, int mw, int nw, int nchunks, int chunks_per_group, double* __restrict__ part) {
-  constexpr int NW = weights<ND>();
+  constexpr int NW = weights<ND>(), TSTAGES = stages<ND>();
   constexpr uint32_t A_TILE = TM * TBK * 2, B_TILE = NT * TBK * 2, STAGE = ND * (A_TILE + B_TILE);
   constexpr uint32_t NCOLS = NW * NT <= 32 ? 32 : NW * NT <= 64 ? 64 : NW * NT <= 128 ? 128 : NW * NT <= 256 ? 256 : 512;
   static_assert(NW * NT <= 512 && NT % 16 == 0, "one accumulator per digit weight");
@@ -365,13 +368,13 @@ struct Shape {
 template <int ND>
 Shape shape_of(int P, int Q, long long n, size_t ws_bytes = SIZE_MAX) {
   Shape s;
-  const int P2 = 2 * P, Q2 = 2 * Q, cap = ND == 6 ? 64 : 128;
+  const int P2 = 2 * P, Q2 = 2 * Q, cap = ND >= 6 ? 64 : 128;
   s.mt = (P2 + TM - 1) / TM;
   s.nt = (Q2 + cap - 1) / cap;
   // tiles of equal width (the MMA takes 128 x NT columns whatever the tile holds)
   s.mw = padded8((P2 + s.mt - 1) / s.mt);
   s.nw = padded8((Q2 + s.nt - 1) / s.nt);
-  s.NT = s.nw <= 16 ? 16 : s.nw <= 48 ? 48 : ND == 6 ? 64 : s.nw <= 80 ? 80 : 128;
+  s.NT = s.nw <= 16 ? 16 : s.nw <= 48 ? 48 : ND >= 6 ? 64 : s.nw <= 80 ? 80 : 128;
   s.nchunks = (int)((n + CHUNK - 1) / CHUNK);
   s.exp_bytes = sizeof(short) * (size_t)s.nchunks * (padded8(P2) + padded8(Q2));
   const size_t per = sizeof(double) * (size_t)P2 * Q2;
@@ -385,6 +388,7 @@ Shape shape_of(int P, int Q, long long n, size_t ws_bytes = SIZE_MAX) {
 
 template <typename R, int ND, int NT>
 cudaError_t launch(const PairBlock<R>& A, const PairBlock<R>& B, const Shape& h, void* ws, cudaStream_t s) {
+  constexpr int TSTAGES = stages<ND>();
   const size_t smem = (size_t)TSTAGES * ND * (TM + NT) * TBK * 2 + 8 * (2 * TSTAGES + 2) + 8 + sizeof(int) * (TM + NT);
   cudaError_t e = allow_dynamic_smem((const void*)k_gram_digits<R, ND, NT>, smem);
   if (e != cudaSuccess) return e;
@@ -413,7 +417,7 @@ cudaError_t gram_digits(const PairBlock<R>& A, const PairBlock<R>& B, double* G_
   if (e != cudaSuccess) return e;
   if (h.NT == 16) e = launch<R, ND, 16>(A, B, h, ws, s);
   else if (h.NT == 48) e = launch<R, ND, 48>(A, B, h, ws, s);
-  else if constexpr (ND == 6) e = launch<R, ND, 64>(A, B, h, ws, s);
+  else if constexpr (ND >= 6) e = launch<R, ND, 64>(A, B, h, ws, s);
   else if (h.NT == 80) e = launch<R, ND, 80>(A, B, h, ws, s);
   else e = launch<R, ND, 128>(A, B, h, ws, s);
   if (e != cudaSuccess) return e;
@@ -436,16 +440,17 @@ bool gram_digits_fits(int P, int Q, long long n, size_t ws_bytes) {
 }
 
 template <typename R>
-cudaError_t gram_pairs_digits(const PairBlock<R>& A, const PairBlock<R>& B, bool fp64, double* G_dev, void* ws,
+cudaError_t gram_pairs_digits(const PairBlock<R>& A, const PairBlock<R>& B, int digits, double* G_dev, void* ws,
                               size_t ws_bytes, cudaStream_t s) {
   if constexpr (sizeof(R) == 8)
-    if (fp64) return gram_digits<R, 6>(A, B, G_dev, ws, ws_bytes, s);
+    if (digits > 4)
+      return digits > 6 ? gram_digits<R, 7>(A, B, G_dev, ws, ws_bytes, s) : gram_digits<R, 6>(A, B, G_dev, ws, ws_bytes, s);
   return gram_digits<R, 4>(A, B, G_dev, ws, ws_bytes, s);
 }
 
-template cudaError_t gram_pairs_digits<float>(const PairBlock<float>&, const PairBlock<float>&, bool, double*, void*,
+template cudaError_t gram_pairs_digits<float>(const PairBlock<float>&, const PairBlock<float>&, int, double*, void*,
                                               size_t, cudaStream_t);
-template cudaError_t gram_pairs_digits<double>(const PairBlock<double>&, const PairBlock<double>&, bool, double*,
+template cudaError_t gram_pairs_digits<double>(const PairBlock<double>&, const PairBlock<double>&, int, double*,
                                                void*, size_t, cudaStream_t);
 
 }  // namespace bdg

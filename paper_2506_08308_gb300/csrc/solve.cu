@@ -371,19 +371,21 @@ class Solver {
   // Grams for which FP32 accuracy suffices -- every Gram of the FP32 phase,
   // and the first pass of the two-pass Gram-Schmidt, whose second pass (FP64)
   // removes what the first leaves -- take four digits per element on the
-  // tensor cores, the others six where gram_digits_pays says so (else
-  // double-float; BDG_GRAM_TC=0: double-float and FP32 SIMT throughout).
+  // tensor cores, the others seven where gram_digits_pays says so (else
+  // double-float; BDG_GRAM_TC=0: double-float and FP32 SIMT throughout).  Not
+  // six: the projected problems amplify what their Grams are off by, and on
+  // coarse grids the residuals of an FP64 solve level off near 1e-10.
   bool tc_ = !getenv("BDG_GRAM_TC") || atoi(getenv("BDG_GRAM_TC")) != 0;
   static constexpr long long TC_MIN_ROWS = 2048;
   bdg_status gram(const PairBlock<R>& A, const PairBlock<R>& B, double* G, bool upper = false,
                   bool fp32_enough = sizeof(R) == 4) {
     if (tc_ && fp32_enough && A.n >= TC_MIN_ROWS && gram_digits_fits(A.cols, B.cols, A.n, gws_bytes_)) {
-      BDG_CUDA_TRY(plan_, gram_pairs_digits<R>(A, B, false, G, gws_, gws_bytes_, s_));
+      BDG_CUDA_TRY(plan_, gram_pairs_digits<R>(A, B, 4, G, gws_, gws_bytes_, s_));
       return BDG_OK;
     }
     if constexpr (sizeof(R) == 8) {
       if (tc_) {
-        BDG_CUDA_TRY(plan_, gram_pairs_fp64(A, B, G, gws_, gws_bytes_, s_, upper));
+        BDG_CUDA_TRY(plan_, gram_pairs_fp64(A, B, G, gws_, gws_bytes_, s_, upper, 7));
         return BDG_OK;
       }
     }
