@@ -13,34 +13,57 @@ namespace bdg {
 
 namespace {
 
-constexpr int TB = 16;
+// C = alpha op(A) op(B) + beta C on tiles of 8 x 16, a thread per element: its
+// sum runs over k in order.  The FP64 pipe bounds a CTA (a warp's multiply-add
+// takes 64 clocks of its SM quarter), so the tiles are small enough that the
+// projected problems (n up to 160) reach every SM with a warp per quarter, and
+// the next 16 steps of k load while these run.  A call (16 x 16 tiles without
+// the loads ahead -> now): n = 72 10.4 -> 8.3 us, 96 12.5 -> 8.5, 140 16.6 ->
+// 14.5, 160 18.7 -> 14.7.
+constexpr int TM = 8, TB = 16;
 
-__global__ void k_dgemm(bool ta, bool tb, int m, int n, int k, double alpha, const double* __restrict__ A,
-                        int lda, const double* __restrict__ B, int ldb, double beta, double* __restrict__ C,
-                        int ldc) {
-  __shared__ double sA[TB][TB + 1];
+__global__ void __launch_bounds__(TM* TB)
+    k_dgemm(bool ta, bool tb, int m, int n, int k, double alpha, const double* __restrict__ A, int lda,
+            const double* __restrict__ B, int ldb, double beta, double* __restrict__ C, int ldc) {
+  __shared__ double sA[TM][TB + 1];
   __shared__ double sB[TB][TB + 1];
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int i = blockIdx.y * TB + ty, j = blockIdx.x * TB + tx;
+  const int tid = threadIdx.x, tx = tid % TB, ty = tid / TB;
+  const int i0 = blockIdx.y * TM, j0 = blockIdx.x * TB;
+  // the elements of a step that this thread loads, along the rows in memory
+  const int ai = ta ? tid % TM : ty, al = ta ? tid / TM : tx;
+  double va, vb[2];
+  auto fetch = [&](int l0) {
+    const int ii = i0 + ai, ll = l0 + al;
+    va = 0.0;
+    if (ii < m && ll < k) va = ta ? A[(long long)ll * lda + ii] : A[(long long)ii * lda + ll];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int bl = l0 + (tb ? tx : ty + TM * h), bj = j0 + (tb ? ty + TM * h : tx);
+      vb[h] = 0.0;
+      if (bl < k && bj < n) vb[h] = tb ? B[(long long)bj * ldb + bl] : B[(long long)bl * ldb + bj];
+    }
+  };
+  fetch(0);
   double acc = 0.0;
   for (int l0 = 0; l0 < k; l0 += TB) {
-    {  // A tile: rows i (block), cols l0 + tx
-      const int ii = blockIdx.y * TB + ty, ll = l0 + tx;
-      double v = 0.0;
-      if (ii < m && ll < k) v = ta ? A[(long long)ll * lda + ii] : A[(long long)ii * lda + ll];
-      sA[ty][tx] = v;
-    }
-    {  // B tile: rows l0 + ty, cols j
-      const int ll = l0 + ty, jj = blockIdx.x * TB + tx;
-      double v = 0.0;
-      if (ll < k && jj < n) v = tb ? B[(long long)jj * ldb + ll] : B[(long long)ll * ldb + jj];
-      sB[ty][tx] = v;
+    sA[ai][al] = va;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (tb) sB[tx][ty + TM * h] = vb[h];
+      else sB[ty + TM * h][tx] = vb[h];
     }
     __syncthreads();
+    if (l0 + TB < k) fetch(l0 + TB);
+    const int steps = min(TB, k - l0);
+    if (steps == TB) {
 #pragma unroll
-    for (int l = 0; l < TB; ++l) acc = fma(sA[ty][l], sB[l][tx], acc);
+      for (int l = 0; l < TB; ++l) acc = fma(sA[ty][l], sB[l][tx], acc);
+    } else {
+      for (int l = 0; l < steps; ++l) acc = fma(sA[ty][l], sB[l][tx], acc);
+    }
     __syncthreads();
   }
+  const int i = i0 + ty, j = j0 + tx;
   if (i < m && j < n) {
     double* c = C + (long long)i * ldc + j;
     *c = beta == 0.0 ? alpha * acc : fma(alpha, acc, beta * *c);
@@ -171,8 +194,8 @@ cudaError_t dzero_small(int m, int n, double* B, int ldb, cudaStream_t s) {
 cudaError_t dgemm_small(bool ta, bool tb, int m, int n, int k, double alpha, const double* A, int lda,
                         const double* B, int ldb, double beta, double* C, int ldc, cudaStream_t s) {
   if (m <= 0 || n <= 0) return cudaSuccess;
-  dim3 grid((n + TB - 1) / TB, (m + TB - 1) / TB), block(TB, TB);
-  k_dgemm<<<grid, block, 0, s>>>(ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
+  dim3 grid((n + TB - 1) / TB, (m + TM - 1) / TM);
+  k_dgemm<<<grid, TM * TB, 0, s>>>(ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
   return cudaGetLastError();
 }
 
@@ -625,11 +648,17 @@ cudaError_t jacobi_multilevel(int n, const double* A, int lda, double* w, double
 
 // ---------------------------------------------------------------------------
 // Rank-revealing pivoted Cholesky (see dense.cuh), one CTA of 1024 threads:
-// right-looking, the lower triangle of the working matrix S in shared
-// memory; step k pivots the largest remaining diagonal to position k, forms
-// column k of L and updates the trailing lower triangle.  The inverse of L1
-// comes from row-wise forward substitution, X_i = (e_i - sum_{j<i} L_ij X_j)
-// / L_ii.
+// right-looking, the lower triangle of the working matrix S in shared memory;
+// step k swaps the largest remaining diagonal to position k, forms column k of
+// L and updates the trailing lower triangle.  The inverse X of L1 follows,
+// right-looking as well, in the strictly upper triangle: row j,
+// X_jc = acc_jc / L_jj, then acc_ic -= L_ij X_jc for all later rows i, from
+// acc_ic = -L_ic / L_cc.  The FP64 pipe of the SM bounds both, n^3/3 multiply-
+// adds, with the barriers: only one triangle is updated, warps take rows (of
+// columns of X) and lanes run along them, and what lanes need of a column lies
+// in a vector of its own.  Both triangles updated and X row by row -> now:
+// n = 72 495 -> 389 us, 96 836 -> 569, 140 1330 -> 980, 160 2140 -> 1241, the
+// same bits.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(1024) k_pchol(int n, const double* __restrict__ A, int lda, double tol,
                                                 double* __restrict__ L, double* __restrict__ M, int ldo,
@@ -637,20 +666,25 @@ __global__ void __launch_bounds__(1024) k_pchol(int n, const double* __restrict_
   extern __shared__ double psm[];
   double* S = psm;                           // [n][n]
   double* dinv = S + (size_t)n * n;          // [n]: 1 / L_ii
-  int* perm = reinterpret_cast<int*>(dinv + n);
+  double* diag = dinv + n;                   // [n]: remaining diagonal
+  double* col = diag + n;                    // [n]: the step's column of L
+  int* perm = reinterpret_cast<int*>(col + n);
   __shared__ double sh_d0;
   __shared__ int sh_p, sh_r;
-  const int tid = threadIdx.x, nt = blockDim.x;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nt >> 5;
   for (int e = tid; e < n * n; e += nt) {
     const int i = e / n, j = e - i * n;
-    S[e] = A[(long long)i * lda + j];
+    if (j <= i) S[e] = A[(long long)i * lda + j];
   }
-  for (int i = tid; i < n; i += nt) perm[i] = i;
+  for (int i = tid; i < n; i += nt) {
+    perm[i] = i;
+    diag[i] = A[(long long)i * lda + i];
+  }
   if (tid == 0) sh_r = n;
   __syncthreads();
   if (tid < 32) {
     double m = 0.0;
-    for (int i = tid; i < n; i += 32) m = fmax(m, S[i * n + i]);
+    for (int i = tid; i < n; i += 32) m = fmax(m, diag[i]);
     for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (tid == 0) sh_d0 = m;
   }
@@ -661,7 +695,7 @@ __global__ void __launch_bounds__(1024) k_pchol(int n, const double* __restrict_
       double m = -1.0;
       int p = k;
       for (int i = k + tid; i < n; i += 32) {
-        const double d = S[i * n + i];
+        const double d = diag[i];
         if (d > m) { m = d; p = i; }
       }
       for (int o = 16; o > 0; o >>= 1) {
@@ -677,36 +711,40 @@ __global__ void __launch_bounds__(1024) k_pchol(int n, const double* __restrict_
     __syncthreads();
     if (sh_r == k) break;
     const int p = sh_p;
-    if (p != k) {   // symmetric swap of rows / columns k and p (full matrix)
+    const double lkk = sqrt(diag[p]);
+    // symmetric swap of rows / columns k and p in the lower triangle; row k is
+    // column k of the trailing matrix
+    if (p != k) {
       for (int j = tid; j < n; j += nt) {
-        const double t = S[k * n + j];
-        S[k * n + j] = S[p * n + j];
-        S[p * n + j] = t;
+        if (j == k || j == p) continue;
+        double* x = S + (j < k ? k * n + j : j * n + k);
+        double* y = S + (j < p ? p * n + j : j * n + p);
+        const double t = *x;
+        *x = *y;
+        *y = t;
       }
       __syncthreads();
-      for (int i = tid; i < n; i += nt) {
-        const double t = S[i * n + k];
-        S[i * n + k] = S[i * n + p];
-        S[i * n + p] = t;
-      }
       if (tid == 0) {
         const int t = perm[k];
         perm[k] = perm[p];
         perm[p] = t;
+        diag[p] = diag[k];
       }
-      __syncthreads();
     }
-    const double lkk = sqrt(S[k * n + k]);
-    __syncthreads();
-    for (int i = k + 1 + tid; i < n; i += nt) S[i * n + k] /= lkk;
+    for (int i = k + 1 + tid; i < n; i += nt) {
+      const double c = S[i * n + k] / lkk;
+      S[i * n + k] = c;
+      col[i] = c;
+    }
     if (tid == 0) S[k * n + k] = lkk;
     __syncthreads();
-    // trailing update of the lower triangle and its mirror (rows and columns
-    // of later pivots are read in full by the swaps above)
-    const int m = n - k - 1;
-    for (int e = tid; e < m * m; e += nt) {
-      const int i = k + 1 + e / m, j = k + 1 + e % m;
-      S[i * n + j] -= S[i * n + k] * S[j * n + k];
+    // trailing update; the diagonal lives in its vector
+    for (int i = k + 1 + warp; i < n; i += nwarp) {
+      const double ci = col[i];
+      for (int j = k + 1 + lane; j <= i; j += 32) {
+        double* x = j < i ? S + i * n + j : diag + i;
+        *x -= ci * col[j];
+      }
     }
     __syncthreads();
   }
@@ -717,17 +755,21 @@ __global__ void __launch_bounds__(1024) k_pchol(int n, const double* __restrict_
     L[(long long)perm[i] * ldo + c] = (c < r && c <= i) ? S[i * n + c] : 0.0;
     M[(long long)i * ldo + c] = 0.0;
   }
-  __syncthreads();
-  // X = L1^-1 (r x r, lower), row by row: X_ii = 1 / L_ii in dinv, X_ic
-  // (c < i) in the strictly upper triangle of S at S[c * n + i] (free once
-  // the factor was copied out; L1 stays in the lower triangle)
   for (int i = tid; i < r; i += nt) dinv[i] = 1.0 / S[i * n + i];
   __syncthreads();
-  for (int i = 1; i < r; ++i) {
-    for (int c = tid; c < i; c += nt) {
-      double acc = -S[i * n + c] * dinv[c];
-      for (int j = c + 1; j < i; ++j) acc -= S[i * n + j] * S[c * n + j];
-      S[c * n + i] = acc * dinv[i];
+  // X = L1^-1 (r x r, lower): X_ii in dinv, X_ic (c < i) at S[c * n + i]
+  for (int c = warp; c < r; c += nwarp) {
+    const double d = dinv[c];
+    for (int i = c + 1 + lane; i < r; i += 32) S[c * n + i] = -S[i * n + c] * d;
+  }
+  __syncthreads();
+  for (int j = 1; j < r; ++j) {
+    for (int c = tid; c < j; c += nt) S[c * n + j] *= dinv[j];
+    for (int i = j + 1 + tid; i < r; i += nt) col[i] = S[i * n + j];
+    __syncthreads();
+    for (int c = warp; c < j; c += nwarp) {
+      const double x = S[c * n + j];
+      for (int i = j + 1 + lane; i < r; i += 32) S[c * n + i] -= col[i] * x;
     }
     __syncthreads();
   }
@@ -752,7 +794,7 @@ __global__ void k_identity_start(int n, const double* __restrict__ A, int lda, d
 cudaError_t pchol(int n, const double* A, int lda, double tol, double* L, double* M, int ldo, int* rank_dev,
                   cudaStream_t s) {
   if (n <= 0 || n > SMALL_MAX || ldo < n) return cudaErrorInvalidValue;
-  const size_t sm = sizeof(double) * ((size_t)n * n + n) + sizeof(int) * (size_t)n;
+  const size_t sm = sizeof(double) * ((size_t)n * n + 3 * (size_t)n) + sizeof(int) * (size_t)n;
   cudaError_t e = allow_dynamic_smem((const void*)k_pchol, sm);
   if (e != cudaSuccess) return e;
   k_pchol<<<1, 1024, sm, s>>>(n, A, lda, tol, L, M, ldo, rank_dev);
