@@ -172,6 +172,7 @@ def source_digest(files):
 
 
 APPLY_SOURCES = ["paper_2506_08308_gb300/csrc/apply_impl.cuh", "paper_2506_08308_gb300/csrc/fft.cuh",
+                 "paper_2506_08308_gb300/csrc/fft2.cuh", "paper_2506_08308_gb300/csrc/apply2_f32.cuh",
                  "paper_2506_08308_gb300/csrc/apply_f32.cu", "paper_2506_08308_gb300/csrc/common.cuh"]
 
 
@@ -684,21 +685,20 @@ def run_ours(args):
                 shares = {"step_device_ms": total / 1000.0, "launches_per_step": n,
                           "kernels": [{"name": k, "launches": c, "ms": t / 1000.0, "share": t / total}
                                       for k, (c, t) in top]}
-                # roofline of the step's dominant kernel, the double-float block
-                # update: its algorithmic FLOPs in the profiled solve (counted by
-                # the library) over its device time in the trace, against the
-                # FP32 SIMT peak divided by the 15 FP32 operations of one
-                # double-float multiply-add
-                upd = per_kernel.get("k_update_df")
+                # roofline of the step's FP64 block updates: their algorithmic
+                # FLOPs in the profiled solve (counted by the library) over
+                # their device time in the trace, against the tensor peak
+                # divided by the 34 digit products of one multiply-add
+                upd = sum(t for k, (_, t) in per_kernel.items() if k.startswith("k_update_d"))
                 fl = plan.stats().get("flops_update_df", 0.0)
-                if upd and upd[1] > 0 and fl > 0:
-                    ach = fl / (upd[1] / 1e6) / 1e12
-                    pk = 152 * 128 * 2 * ((clocks or {}).get("sm_max_mhz") or 2070.0) * 1e6 / 1e12 / 15.0
-                    dominant = {"kernel": "k_update_df (FP64 block update in double-float)", "share": upd[1] / total,
+                if upd > 0 and fl > 0:
+                    ach = fl / (upd / 1e6) / 1e12
+                    pk = measured_peaks()[0]["bf16_tflops"] / 34.0
+                    dominant = {"kernel": "k_update_digits, k_update_df (FP64 block updates)", "share": upd / total,
                                 "bound": "alu", "achieved": ach, "peak": pk, "unit": "TFLOP/s", "frac": ach / pk,
                                 "traffic": None,
-                                "peak_kind": "derived: 152 SMs x 128 FP32 lanes x 2 x SM clock / 15 FP32 "
-                                             "operations per double-float multiply-add"}
+                                "peak_kind": "derived: measured dense 16-bit tensor rate / 34 digit products "
+                                             "per FP64 multiply-add"}
         except Exception as exc:  # noqa: BLE001 -- auxiliary evidence only
             launches, shares = None, {"error": f"{type(exc).__name__}: {exc}"[:300]}
 
