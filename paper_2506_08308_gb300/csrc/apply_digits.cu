@@ -380,12 +380,14 @@ __global__ void __launch_bounds__(THREADS, 1)
 // y = C x: the pointwise coupling of all six components, one thread per node
 // and up to VECS vectors, for which the node's 21 coefficients are formed
 // once.  In the UV form A u + B v and B u + A v come from P f and M g with f =
-// u + v, g = u - v, P = (A + B) / 2, M = (A - B) / 2.
+// u + v, g = u - v, P = (A + B) / 2, M = (A - B) / 2.  The CTAs of all nodes,
+// then of all groups of vectors, lie along x (gridDim.y ends at 65535 groups,
+// about a million vectors); node_bits: log2 of the node blocks.
 constexpr int VECS = 16;
 __global__ void __launch_bounds__(128) k_couple(const double2* __restrict__ x, double2* __restrict__ y, long long npts,
-                                                int nvec, const dquad* __restrict__ phiv, Coupling<double> cp, int mode) {
-  const long long i = (long long)blockIdx.x * 128 + threadIdx.x;
-  if (i >= npts) return;
+                                                int node_bits, int nvec, const dquad* __restrict__ phiv,
+                                                Coupling<double> cp, int mode) {
+  const long long i = (long long)(blockIdx.x & ((1u << node_bits) - 1)) * 128 + threadIdx.x;
   Sym3<double> A, B;
   coupling_blocks<double>(phiv[i], cp, A, B);
   Sym3<double> P = sym_add(A, B, 1.0), M = sym_add(A, B, -1.0);
@@ -396,7 +398,7 @@ __global__ void __launch_bounds__(128) k_couple(const double2* __restrict__ x, d
     half(P);
     half(M);
   }
-  const int v0 = blockIdx.y * VECS, v1 = min(nvec, v0 + VECS);
+  const int v0 = (int)(blockIdx.x >> node_bits) * VECS, v1 = min(nvec, v0 + VECS);
   for (int v = v0; v < v1; ++v) {
     const double2* p = x + (long long)v * 6 * npts + i;
     double2* o = y + (long long)v * 6 * npts + i;
@@ -484,8 +486,9 @@ cudaError_t axis_digits_table(int n, uint8_t** out, int* kexp, cudaStream_t s) {
 }
 
 cudaError_t couple_launch(const ApplyArgs<double>& g, cudaStream_t s) {
-  const dim3 grid((unsigned)((g.grid->npts + 127) / 128), (unsigned)((g.nvec + VECS - 1) / VECS));
-  k_couple<<<grid, 128, 0, s>>>(g.x, g.y, g.grid->npts, g.nvec, g.phiv, g.cp, g.mode);
+  const long long nodes = g.grid->npts / 128;   // (an axis of 128 or 256 points: a power of two, no remainder)
+  const long long ctas = nodes * ((g.nvec + VECS - 1LL) / VECS);
+  k_couple<<<(unsigned)ctas, 128, 0, s>>>(g.x, g.y, g.grid->npts, log2i(nodes), g.nvec, g.phiv, g.cp, g.mode);
   return cudaGetLastError();
 }
 
