@@ -23,11 +23,11 @@
 // 2.7e-16 (128), noise under a Gaussian 2.3e-16 / 2.9e-16, smooth functions
 // (whose result is a small difference) 1.1e-13 / 1.9e-13.
 //
-// 256^2, 32 vectors, UV: 3097 us with FFTs -> 995 us: 370 us per axis (a tile
+// 256^2, 32 vectors, UV: 3097 us with FFTs -> 1052 us: 370 us per axis (a tile
 // of 64 real lines takes 14 us of MMAs, each bound by its 6 KB of operands at
 // 128 bytes per clock, and about 20 of integer work at 1.7 instructions a
 // clock, one after the other: tensor memory and shared memory hold one block
-// at a time), 256 us of coupling at 88 % of the FP64 pipe.
+// at a time), 310 us of coupling, 240 of which are the FP64 pipe's multiply-adds.
 //
 // One CTA of sixteen warps per SM, 32 complex (64 real) lines a tile: the
 // warps load, fold and cut the digits of a block of 128 x 64 values (MMA B
@@ -377,56 +377,60 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (warp == 0) tmem_free(tmem, 512);
 }
 
+// acc + row r of m times x
+__device__ __forceinline__ double2 row_fma(double m0, double m1, double m2, const double2 (&x)[3], double2 acc) {
+  return cfma(x[2], m2, cfma(x[1], m1, cfma(x[0], m0, acc)));
+}
+__device__ __forceinline__ void mul3_add(const Sym3<double>& m, const double2 (&x)[3], double2 (&y)[3]) {
+  y[0] = row_fma(m.d0, m.o01, m.o02, x, y[0]);
+  y[1] = row_fma(m.o01, m.d1, m.o12, x, y[1]);
+  y[2] = row_fma(m.o02, m.o12, m.d2, x, y[2]);
+}
+
 // y = C x: the pointwise coupling of all six components, one thread per node
 // and up to VECS vectors, for which the node's 21 coefficients are formed
-// once.  In the UV form A u + B v and B u + A v come from P f and M g with f =
-// u + v, g = u - v, P = (A + B) / 2, M = (A - B) / 2.  The CTAs of all nodes,
-// then of all groups of vectors, lie along x (gridDim.y ends at 65535 groups,
-// about a million vectors); node_bits: log2 of the node blocks.
+// once.  The UV form sums A u + B v and B u + A v as they stand: half the
+// products would do with (A + B) / 2 and (A - B) / 2 on u + v and u - v, but the
+// small B u would then be a difference of two terms of the size of A u.  The
+// CTAs of all nodes, then of all groups of vectors, lie along x (gridDim.y ends
+// at 65535 groups, about a million vectors); node_bits: log2 of the node blocks.
 constexpr int VECS = 16;
 __global__ void __launch_bounds__(128) k_couple(const double2* __restrict__ x, double2* __restrict__ y, long long npts,
                                                 int node_bits, int nvec, const dquad* __restrict__ phiv,
                                                 Coupling<double> cp, int mode) {
   const long long i = (long long)(blockIdx.x & ((1u << node_bits) - 1)) * 128 + threadIdx.x;
-  Sym3<double> A, B;
+  Sym3<double> A, B;   // UV: the blocks; FG: A + B and A - B
   coupling_blocks<double>(phiv[i], cp, A, B);
-  Sym3<double> P = sym_add(A, B, 1.0), M = sym_add(A, B, -1.0);
-  if (mode == BDG_UV) {
-    auto half = [](Sym3<double>& m) {
-      m.d0 *= 0.5; m.d1 *= 0.5; m.d2 *= 0.5; m.o01 *= 0.5; m.o12 *= 0.5; m.o02 *= 0.5;
-    };
-    half(P);
-    half(M);
+  if (mode != BDG_UV) {
+    const Sym3<double> P = sym_add(A, B, 1.0);
+    B = sym_add(A, B, -1.0);
+    A = P;
   }
   const int v0 = (int)(blockIdx.x >> node_bits) * VECS, v1 = min(nvec, v0 + VECS);
   for (int v = v0; v < v1; ++v) {
     const double2* p = x + (long long)v * 6 * npts + i;
     double2* o = y + (long long)v * 6 * npts + i;
-    double2 a[3], b[3];
+    double2 a[3], b[3], f[3], g[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       a[c] = p[c * npts];
       b[c] = p[(3 + c) * npts];
+      f[c] = g[c] = make_double2(0.0, 0.0);
     }
+    mul3_add(A, a, f);
     if (mode == BDG_UV) {
+      mul3_add(B, b, f);
+      mul3_add(B, a, g);
+      mul3_add(A, b, g);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const double2 f = a[c] + b[c], g = a[c] - b[c];
-        a[c] = f;
-        b[c] = g;
-      }
+      for (int c = 0; c < 3; ++c) g[c] = make_double2(-g[c].x, -g[c].y);
+    } else {
+      mul3_add(B, b, g);
     }
-    double2 f[3], g[3];
-    f[0] = sym3_row0(P, a[0], a[1], a[2]);
-    f[1] = sym3_row1(P, a[0], a[1], a[2]);
-    f[2] = sym3_row2(P, a[0], a[1], a[2]);
-    g[0] = sym3_row0(M, b[0], b[1], b[2]);
-    g[1] = sym3_row1(M, b[0], b[1], b[2]);
-    g[2] = sym3_row2(M, b[0], b[1], b[2]);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      o[c * npts] = mode == BDG_UV ? f[c] + g[c] : f[c];
-      o[(3 + c) * npts] = mode == BDG_UV ? g[c] - f[c] : g[c];
+      o[c * npts] = f[c];
+      o[(3 + c) * npts] = g[c];
     }
   }
 }

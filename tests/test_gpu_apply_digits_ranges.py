@@ -33,3 +33,33 @@ def test_more_than_a_million_vectors():
     for i in range(0, nvec, part):
         assert torch.equal(y[i:i + part], plan.apply(x[i:i + part], bdg.UV)), i
     plan.close()
+
+
+@pytest.mark.parametrize("n,nvec", [((256, 256), 2), ((128, 8, 128), 2), ((256,), 350)])
+def test_small_coupling_beside_a_large_one(n, nvec):
+    """UV form with v = 0: the last three components are -B u alone, with a
+    relative accuracy of the sum of |B u|'s three terms: 8 units of 2^-53 for
+    B's entries (six roundings at most) and the products."""
+    torch = need_torch_cuda()
+    from paper_2506_08308_gb300 import bdg
+    w, op, plan = _setup(n)
+    x = synth.random_block(w, nvec, seed=5)
+    x[:, 3:] = 0.0
+    y = plan.apply(torch.from_numpy(x).cuda(), bdg.UV).cpu().numpy()[:, 3:]
+    a, b, c = (synth.initial_spinor(w) * 0.3).reshape(3, -1).astype(np.longdouble)
+    bn, bs = np.longdouble(w.beta_n), np.longdouble(w.beta_s)
+    B = [[(bn + bs) * a * a, (bn + bs) * a * b, bn * a * c + bs * (b * b - a * c)],
+         [(bn + bs) * a * b, bn * b * b + 2 * bs * a * c, (bn + bs) * b * c],
+         [bn * a * c + bs * (b * b - a * c), (bn + bs) * b * c, (bn + bs) * c * c]]
+    # (terms of an entry before they cancel)
+    S = [[abs(e) for e in r] for r in B]
+    S[0][2] = S[2][0] = abs(bn * a * c) + abs(bs) * (b * b + abs(a * c))
+    S[1][1] = abs(bn) * b * b + 2 * abs(bs * a * c)
+    for j in range(3):
+        for part in ("real", "imag"):
+            u = getattr(x[:, :3], part).astype(np.longdouble)
+            ref = -sum(B[j][k] * u[:, k] for k in range(3))
+            size = sum(S[j][k] * abs(u[:, k]) for k in range(3))
+            err = abs(getattr(y[:, j], part) - ref) / size
+            assert err.max() < 8 * 2.0 ** -53, (j, part, err.max())
+    plan.close()
