@@ -95,15 +95,16 @@ __device__ __forceinline__ long long weigh(const float (&c)[NW]) {
   return hi + e + ((f + 128) >> 8);
 }
 
-// int64 to double (round to nearest, away from zero in the ties) without the
-// FP64 pipe; |v| < 2^62
-__device__ __forceinline__ double to_double(long long v) {
+// v 2^(top - TOP) as a double (round to nearest, away from zero in the ties)
+// without the FP64 pipe; |v| < 2^62
+constexpr int TOP = 1085;
+__device__ __forceinline__ double to_double(long long v, int top) {
   const int s = (int)(v >> 63);
   const unsigned long long m = (unsigned long long)((v ^ (long long)s) - (long long)s);
   const int lz = __clzll((long long)m);  // 2 .. 64
   const unsigned long long n = (m << (lz & 63)) + 0x400;        // leading bit at 63, half a unit of bit 11 added
-  unsigned long long bits = ((unsigned long long)(unsigned)(1085 - lz) << 52) + (n >> 11);  // (the leading bit adds one)
-  if (n < 0x400ull) bits = (unsigned long long)(unsigned)(1087 - lz) << 52;                 // a carry out of bit 63
+  unsigned long long bits = ((unsigned long long)(unsigned)(top - lz) << 52) + (n >> 11);  // (the leading bit adds one)
+  if (n < 0x400ull) bits = (unsigned long long)(unsigned)(top + 2 - lz) << 52;                 // a carry out of bit 63
   if (m == 0) bits = 0;
   return __longlong_as_double((long long)(bits | ((unsigned long long)(unsigned)s << 63 & 0x8000000000000000ull)));
 }
@@ -124,7 +125,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint64_t* done = empty + STAGES;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
   int* bad = reinterpret_cast<int*>(tmem_slot + 1);          // a wait ran out: the results become NaN
-  int* ex = reinterpret_cast<int*>(tmem_slot + 2);          // [LINES] largest exponents
+  unsigned* ex = reinterpret_cast<unsigned*>(tmem_slot + 2);  // [LINES] largest magnitudes
   double* sc = reinterpret_cast<double*>(ex + LINES);       // [LINES] scale of the result
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
 
@@ -184,16 +185,16 @@ __global__ void __launch_bounds__(THREADS, 1)
         for (int b = 0; b < NB; ++b) v[q][l][b] = p[(64 * q + BLK * b) * st];
     }
     __syncthreads();
-    // largest exponent of every real line
+    // largest magnitude of every real line
 #pragma unroll
     for (int l = 0; l < 4; ++l) {
-      int mr = 0, mi = 0;
+      unsigned mr = 0, mi = 0;
 #pragma unroll
       for (int q = 0; q < 2; ++q)
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
-          mr = max(mr, exponent_of(v[q][l][b].x));
-          mi = max(mi, exponent_of(v[q][l][b].y));
+          mr = max(mr, magnitude(v[q][l][b].x));
+          mi = max(mi, magnitude(v[q][l][b].y));
         }
       if (st == 1) {
         mr = __reduce_max_sync(0xffffffffu, mr);
@@ -211,8 +212,13 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
     }
     __syncthreads();
+    // tiny lines (digits.cuh) among the tile's are cut times 2^GROW; their
+    // scales hold that factor too, and the integer results its inverse
+    const bool rare = __any_sync(0xffffffffu, is_tiny<double>(ex[lane]) || is_tiny<double>(ex[lane + 32]));
+    auto tiny = [&](int line) { return rare && is_tiny<double>(ex[line]); };
+    auto top_of = [&](int line) { return tiny(line) ? TOP - Tiny<double>::GROW : TOP; };
     if (tid < LINES) {
-      const int e = ex[tid];
+      const int e = biased_exponent<double>(ex[tid]) + (tiny(tid) ? Tiny<double>::GROW : 0);
       const long long ln = min(tile * (LINES / 2) + tid / 2, nlines - 1);
       const double sg = mode == BDG_UV && (int)((ln >> comp_bits) % 6) >= 3 ? -kfac : kfac;
       sc[tid] = e >= 2047 ? (double)NAN : e == 0 ? 0.0 : scalbn(sg, e + kexp - 1076);
@@ -221,7 +227,17 @@ __global__ void __launch_bounds__(THREADS, 1)
     long long X[NB][2][4][2];
 #pragma unroll
     for (int l = 0; l < 4; ++l) {
-      const int er = ex[8 * g + 2 * l] << 20, ei = ex[8 * g + 2 * l + 1] << 20;
+      const int lr = 8 * g + 2 * l, li = lr + 1;
+      int er = (int)ex[lr], ei = (int)ex[li];
+      auto grow = [&](int& e, auto part) {
+        e = (biased_exponent<double>(e) + Tiny<double>::GROW) << 20;
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+          for (int b = 0; b < NB; ++b) part(v[q][l][b]) *= Tiny<double>::FACTOR;
+      };
+      if (tiny(lr)) grow(er, [](double2& z) -> double& { return z.x; });
+      if (tiny(li)) grow(ei, [](double2& z) -> double& { return z.y; });
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         long long r[NB], i[NB];
@@ -330,15 +346,17 @@ __global__ void __launch_bounds__(THREADS, 1)
         const double sr = *bad ? (double)NAN : sc[cg + q], si = *bad ? (double)NAN : sc[cg + q + 1];
         double2 u = *p;
         double2 w = NB == 2 ? p[BLK] : u;
-        *p = make_double2(fma(to_double(c0[q]), sr, u.x), fma(to_double(c0[q + 1]), si, u.y));
+        const int tr = top_of(cg + q), ti = top_of(cg + q + 1);
+        *p = make_double2(fma(to_double(c0[q], tr), sr, u.x), fma(to_double(c0[q + 1], ti), si, u.y));
         if constexpr (NB == 2)
-          p[BLK] = make_double2(fma(to_double(c1[q]), sr, w.x), fma(to_double(c1[q + 1]), si, w.y));
+          p[BLK] = make_double2(fma(to_double(c1[q], tr), sr, w.x), fma(to_double(c1[q + 1], ti), si, w.y));
       }
     } else {        // through shared memory, where the digits were: lanes to neighbouring lines
       long long* stage = reinterpret_cast<long long*>(xd);   // [128 points][32 lines][re, im], lines swizzled
       const bool on = tile * (LINES / 2) + lane < nlines;
       double2* p = y + line_base(tile, lane);
       const double sr = *bad ? (double)NAN : sc[2 * lane], si = *bad ? (double)NAN : sc[2 * lane + 1];
+      const int tr = top_of(2 * lane), ti = top_of(2 * lane + 1);
 #pragma unroll
       for (int h = 0; h < NB; ++h) {
         if (h) __syncthreads();
@@ -359,7 +377,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             for (int r = 0; r < RB; ++r) {
               const int m = n + 16 * r;
               const longlong2 c = *reinterpret_cast<const longlong2*>(stage + 2 * (m * 32 + (lane ^ (m & 31))));
-              p[(h * BLK + m) * st] = make_double2(fma(to_double(c.x), sr, u[r].x), fma(to_double(c.y), si, u[r].y));
+              p[(h * BLK + m) * st] = make_double2(fma(to_double(c.x, tr), sr, u[r].x), fma(to_double(c.y, ti), si, u[r].y));
             }
           }
         }

@@ -90,23 +90,49 @@ __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.
 // ---------------------------------------------------------------------------
 // fixed point
 // ---------------------------------------------------------------------------
-// Biased FP64 exponent of |x| (0: zero or subnormal, taken as zero; 2047:
-// infinity or NaN), of either type.
-__device__ __forceinline__ int exponent_of(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
-__device__ __forceinline__ int exponent_of(float x) {
-  const int e = (__float_as_int(x) >> 23) & 0xFF;
-  return e == 0 ? 0 : e == 0xFF ? 2047 : e + 896;
+// An integer in the order of |x|, zero for zero only; an FP64 value's exponent
+// field is in its bits 20..30, an FP32 value's in 23..30.
+__device__ __forceinline__ unsigned magnitude(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7FFFFFFFu) | min((unsigned)__double2loint(x), 1u);
+}
+__device__ __forceinline__ unsigned magnitude(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
+// Biased FP64 exponent of the largest value of a column from its magnitude: 0
+// for zeros only, 1 (897 for FP32) where all are subnormal, 2047 for an
+// infinity or NaN.
+template <typename R>
+__device__ __forceinline__ int biased_exponent(unsigned m) {
+  if (m == 0) return 0;
+  if constexpr (sizeof(R) == 8) return max((int)(m >> 20), 1);
+  return m >= 0x7F800000u ? 2047 : max((int)(m >> 23), 1) + 896;
+}
+// Zeros and subnormals have no implicit bit, which to_fixed sets for all: it
+// falls below the last digit unless the column's largest value is very small.
+// Such a column (magnitude below LIMIT) is multiplied by 2^GROW first.
+template <typename R> struct Tiny;
+template <> struct Tiny<double> {
+  static constexpr unsigned LIMIT = 128u << 20;
+  static constexpr int GROW = 200;
+  static constexpr double FACTOR = 0x1p200;
+};
+template <> struct Tiny<float> {
+  static constexpr unsigned LIMIT = 64u << 23;
+  static constexpr int GROW = 64;
+  static constexpr float FACTOR = 0x1p64f;
+};
+template <typename R>
+__device__ __forceinline__ bool is_tiny(unsigned m) {
+  return m - 1u < Tiny<R>::LIMIT - 1u;   // (a column of zeros is not)
 }
 
 // Fixed point of x relative to 2^(emax - 1022), emax the largest biased
-// exponent of its column.  e20 holds emax in bits 20..31 (the bits below may
-// be anything).
+// exponent of its column, which is not a tiny one.  e20 holds emax in bits
+// 20..30 (the bits below may be anything, as in a magnitude).
 // ND = 6, 7: the value's 53 bits with two more below, |X| < 2^55, x = X
 //   2^(emax - 1077), as seven bytes; six digits leave out the lowest byte,
 //   which the bias of 0x80 per byte turns into rounding to nearest.
 // ND = 4: |X| < 2^30, x = X 2^(emax - 1052), rounded down.
-// Values whose exponent is zero come out as at most one unit unless emax is
-// zero as well; the caller takes such a column as zero.
+// Zeros and subnormals come out as at most one unit.  A column of zeros has
+// emax = 0, whose X is finite and means nothing: the caller leaves it out.
 template <int ND> struct Fixed { typedef long long I; };
 template <> struct Fixed<4> { typedef int I; };
 

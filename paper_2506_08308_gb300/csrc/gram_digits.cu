@@ -52,34 +52,40 @@ template <int ND> constexpr int weights() { return ND >= 6 ? ND + 1 : ND; }
 template <int ND> constexpr int stages() { return ND == 7 ? 2 : 3; }
 inline int padded8(int cols) { return (cols + 7) / 8 * 8; }
 
-// exps[chunk * ld + 2 c + part]: largest biased exponent of the column's real
-// (imaginary) parts in the chunk; one warp per chunk and complex column, the
-// columns up to ld (2 cols rounded up to 8) are zero
+// A column's entry in the table of exponents: the biased exponent of its largest
+// value in the chunk, with TINY_BIT where that is a tiny one (digits.cuh).
+constexpr int TINY_BIT = 0x1000;
+__device__ __forceinline__ int exponent_in(int entry) { return entry & (TINY_BIT - 1); }
+
+// exps[chunk * ld + 2 c + part]: the entries of the column's real and imaginary
+// parts; one warp per chunk and complex column, the columns up to ld (2 cols
+// rounded up to 8) are zero
 template <typename R>
 __global__ void __launch_bounds__(256) k_col_exp(PairBlock<R> X, int nchunks, int ld, short* __restrict__ exps) {
   typedef typename CT<R>::T T;
   const int warp = (int)((blockIdx.x * 256LL + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   const int c = warp / nchunks, chunk = warp - c * nchunks;
   if (2 * c >= ld) return;
+  auto entry = [](unsigned m) { return biased_exponent<R>(m) | (is_tiny<R>(m) ? TINY_BIT : 0); };
   if (c >= X.cols) {
     if (lane == 0) *reinterpret_cast<short2*>(exps + (long long)chunk * ld + 2 * c) = make_short2(0, 0);
     return;
   }
   const T* p = X.p + (long long)c * X.ld + (long long)chunk * CHUNK;
   const int rows = (int)min((long long)CHUNK, X.n - (long long)chunk * CHUNK);
-  int ex = 0, ey = 0;
+  unsigned mx = 0, my = 0;
 #pragma unroll
   for (int k = 0; k < CHUNK / 32; ++k) {
     const int r = lane + 32 * k;
     if (r < rows) {
       const T v = p[r];
-      ex = max(ex, exponent_of(v.x));
-      ey = max(ey, exponent_of(v.y));
+      mx = max(mx, magnitude(v.x));
+      my = max(my, magnitude(v.y));
     }
   }
-  ex = __reduce_max_sync(0xffffffffu, ex);
-  ey = __reduce_max_sync(0xffffffffu, ey);
-  if (lane == 0) *reinterpret_cast<short2*>(exps + (long long)chunk * ld + 2 * c) = make_short2((short)ex, (short)ey);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  my = __reduce_max_sync(0xffffffffu, my);
+  if (lane == 0) *reinterpret_cast<short2*>(exps + (long long)chunk * ld + 2 * c) = make_short2((short)entry(mx), (short)entry(my));
 }
 
 // 2^e as a float for e <= 0, 0 below the normal range
@@ -120,8 +126,17 @@ struct RowTask {
 };
 // digits of eight real columns at one row: 16 bytes per digit tile
 template <typename R, int ND>
-__device__ __forceinline__ void store_task(const RowTask<R>& x, uint8_t* base, uint32_t tile_bytes) {
-  const unsigned e[4] = {x.ev.x, x.ev.y, x.ev.z, x.ev.w};
+__device__ __forceinline__ void store_task(RowTask<R>& x, uint8_t* base, uint32_t tile_bytes) {
+  unsigned e[4] = {x.ev.x, x.ev.y, x.ev.z, x.ev.w};
+  constexpr unsigned LO = TINY_BIT, HI = (unsigned)TINY_BIT << 16;
+  if ((e[0] | e[1] | e[2] | e[3]) & (LO | HI)) {   // (all lanes have the same columns)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (e[q] & LO) x.v[q].x *= Tiny<R>::FACTOR;
+      if (e[q] & HI) x.v[q].y *= Tiny<R>::FACTOR;
+      e[q] += (e[q] & LO ? Tiny<R>::GROW : 0) + (e[q] & HI ? Tiny<R>::GROW << 16 : 0);
+    }
+  }
   uint32_t d[4][ND];
 #pragma unroll
   for (int q = 0; q < 4; ++q)
@@ -181,7 +196,7 @@ __global__ void __launch_bounds__(TTHREADS, 1)
     const short* e = isA ? expA : expB;
     int m = 0;
     if (col < (isA ? i1 : j1))
-      for (int ch = ch0; ch < ch1; ++ch) m = max(m, (int)e[(long long)ch * ld + col]);
+      for (int ch = ch0; ch < ch1; ++ch) m = max(m, exponent_in(e[(long long)ch * ld + col]));
     (isA ? ra : rb)[isA ? c : c - TM] = m;
   }
   tc_fence_before();
@@ -245,8 +260,8 @@ __global__ void __launch_bounds__(TTHREADS, 1)
       if (!mma_wait(acc_full, (uint32_t)(chunk & 1))) lost = true;
       tc_fence_after();
       const int ch = ch0 + chunk;
-      // (a column without a normal number in the chunk counts as zero)
-      const int xa = i0 + row < i1 ? (int)expA[(long long)ch * ldea + i0 + row] : 0;
+      // (a column of zeros in the chunk has no digits that mean anything)
+      const int xa = i0 + row < i1 ? exponent_in(expA[(long long)ch * ldea + i0 + row]) : 0;
       const float fa = xa ? pow2_neg(xa - ra[row]) : 0.f;
 #pragma unroll
       for (int c0 = 0; c0 < NQ; c0 += 4) {
@@ -256,7 +271,7 @@ __global__ void __launch_bounds__(TTHREADS, 1)
         int e[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const int xb = j0 + jq + c0 + q < j1 ? (int)expB[(long long)ch * ldeb + j0 + jq + c0 + q] : 0;
+          const int xb = j0 + jq + c0 + q < j1 ? exponent_in(expB[(long long)ch * ldeb + j0 + jq + c0 + q]) : 0;
           e[q] = xb ? xb - rb[jq + c0 + q] : -4096;
         }
         tmem_ld_wait();

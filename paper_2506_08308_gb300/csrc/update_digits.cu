@@ -52,11 +52,13 @@ __global__ void __launch_bounds__(KMAX) k_update_table(const double* __restrict_
   if (k == 0) emax = 0;
   __syncthreads();
   const double v = j < Q2 && k < K ? alpha * C[(long long)k * ldc + j] : 0.0;
-  atomicMax(&emax, exponent_of(v));
+  // (a subnormal coefficient counts as zero, and a zero as no value: no TINY case)
+  const int ev = (__double2hiint(v) >> 20) & 0x7FF;
+  atomicMax(&emax, ev);
   __syncthreads();
   if (k == 0) exps[j] = (short)emax;
   if (k >= kpad) return;
-  const long long X = emax > 0 && exponent_of(v) > 0 ? to_fixed<ND>(v, emax << 20) : 0;
+  const long long X = ev > 0 ? to_fixed<ND>(v, emax << 20) : 0;
   const unsigned long long u = (unsigned long long)X + 0x80808080808080ull;
   const int st = k / KC, k8 = k % KC / 8;
   __half* o = out + (size_t)st * ND * N * KC + (k8 * (N / 8) + j / 8) * 64 + (k % 8) * 8 + j % 8;
@@ -108,8 +110,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint64_t* done = empty + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
   int* bad = reinterpret_cast<int*>(tmem_slot + 1);
-  int* er = bad + 1;                                               // [ROWS]
-  int* ecs = er + ROWS;                                            // [N]
+  unsigned* er = reinterpret_cast<unsigned*>(bad + 1);             // [ROWS] largest magnitudes
+  int* ecs = reinterpret_cast<int*>(er + ROWS);                                            // [N]
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   if (warp == 0) tmem_alloc(tmem_slot, NCOLS);
   if (tid == 0) {
@@ -135,7 +137,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     const long long r = tile * ROWS + row;
     const bool in = r < A.n;
     double2 v[GROUPS][4];
-    int m = 0;
+    unsigned m = 0;
 #pragma unroll
     for (int s = 0; s < GROUPS; ++s)
 #pragma unroll
@@ -149,10 +151,20 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
     for (int s = 0; s < GROUPS; ++s)
 #pragma unroll
-      for (int l = 0; l < 4; ++l) m = max(m, max(exponent_of(v[s][l].x), exponent_of(v[s][l].y)));
+      for (int l = 0; l < 4; ++l) m = max(m, max(magnitude(v[s][l].x), magnitude(v[s][l].y)));
     atomicMax(&er[row], m);
     __syncthreads();
-    const int e20 = er[row] << 20;
+    int e20 = (int)er[row];
+    if (is_tiny<double>(e20)) {
+      e20 = (biased_exponent<double>(e20) + Tiny<double>::GROW) << 20;
+#pragma unroll
+      for (int s = 0; s < GROUPS; ++s)
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+          v[s][l].x *= Tiny<double>::FACTOR;
+          v[s][l].y *= Tiny<double>::FACTOR;
+        }
+    }
 #pragma unroll
     for (int s = 0; s < GROUPS; ++s) {
       if (s >= nst) break;
@@ -204,7 +216,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     constexpr int NQ = N / 4;
     const int quarter = warp & 3, jq = (warp >> 2) * NQ, orow = 32 * quarter + lane;
     const long long ro = tile * ROWS + orow;
-    const int eo = er[orow];
+    const int eo = biased_exponent<double>(er[orow]);
     if (lost) *bad = 1;
     __syncthreads();
 #pragma unroll

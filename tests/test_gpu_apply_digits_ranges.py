@@ -63,3 +63,29 @@ def test_small_coupling_beside_a_large_one(n, nvec):
             err = abs(getattr(y[:, j], part) - ref) / size
             assert err.max() < 8 * 2.0 ** -53, (j, part, err.max())
     plan.close()
+
+
+@pytest.mark.parametrize("n,nvec", [((128,), 350), ((256,), 350), ((128, 64), 6), ((256, 32), 9)])
+@pytest.mark.parametrize("k", [-960, -1000, -1030])
+def test_lines_of_very_small_values(n, nvec, k):
+    """Lines down to subnormal values, with zeros between them: x 2^k gives the
+    result 2^k times that of x, to 2^-54 of a line's largest value and to
+    2^-1074 (the spacing of subnormal numbers, at which the passes that stay
+    FFTs and the coupling round) times the l1 norm N^2 / 4 of an axis' kernel
+    (kappa < 1); four times that for the roundings one after another."""
+    torch = need_torch_cuda()
+    from paper_2506_08308_gb300 import bdg
+    w, op, plan = _setup(n)
+    x = synth.random_block(w, nvec, seed=6)
+    x[:, :, ::3] = 0.0
+    x[::4] *= 1e-12                  # lines of other sizes in the same tile
+    x[1] = 0.0
+    x = np.ldexp(np.ldexp(x.view(np.float64), k), -k).view(np.complex128)   # (what survives as a subnormal)
+    xk = np.ldexp(x.view(np.float64), k).view(np.complex128)
+    for mode in (bdg.UV, bdg.FG):
+        y = plan.apply(torch.from_numpy(x).cuda(), mode).cpu().numpy()
+        yk = plan.apply(torch.from_numpy(xk).cuda(), mode).cpu().numpy()
+        yk = np.ldexp(yk.view(np.float64), -k).view(np.complex128)
+        tol = sum(m * m for m in n) * (2.0 ** -56 * np.abs(x).max(axis=(1, 2)) + 2.0 ** (-1074 - k))
+        assert np.all(np.abs(yk - y).max(axis=(1, 2)) <= tol), np.abs(yk - y).max(axis=(1, 2)) / tol
+    plan.close()
