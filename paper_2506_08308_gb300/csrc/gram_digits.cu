@@ -8,10 +8,15 @@
 // against which its values are cut into digits; within a chunk the products
 // of each digit weight add up in one FP32 accumulator, exactly for the four
 // leading weights (256 rows x 4 pairs x 2^14 = 2^24), to 2^-24 of a part
-// below 2^-32 of the result for the others.  After a chunk the
-// accumulators are read back and added, error-free down to the second float,
-// to a double-float sum per output in registers; the CTA writes its sum as
-// FP64, and the CTAs' partial sums are added in FP64 in a fixed order.
+// below 2^-32 of the result for the others.  After a chunk the accumulators
+// are read back.  FP64 accuracy: the weights are put together in a 64-bit
+// integer, in units of 2^-54 of the product of the columns' largest values, and
+// added to an FP64 sum per output in registers.  (In one double-float sum, the
+// weights from the fourth on in one float, what 256 rows lost was 2^-47 of that
+// product, and of 288 FP64 solves of 64^2 problems 38 levelled off above their
+// tolerance of 1e-10; 18 with double-float Grams, one now.)  FP32 accuracy: the
+// leading three weights error-free into a double-float sum.  The CTA writes its
+// sums as FP64, and the CTAs' partial sums are added in FP64 in a fixed order.
 //
 // Why: a double-float multiply-add is 15 FP32 instructions, so the same
 // contraction in double-float is bound by the FP32 pipe at 5 TFLOP/s (and
@@ -88,6 +93,18 @@ __global__ void __launch_bounds__(256) k_col_exp(PairBlock<R> X, int nchunks, in
   if (lane == 0) *reinterpret_cast<short2*>(exps + (long long)chunk * ld + 2 * c) = make_short2((short)entry(mx), (short)entry(my));
 }
 
+// v 2^(e - 40) as a double for |v| < 2^62 and e <= 0 (0 for e < -900), rounded to
+// nearest, without the FP64 pipe
+__device__ __forceinline__ double chunk_value(long long v, int e) {
+  const int s = (int)(v >> 63);
+  const unsigned long long m = (unsigned long long)((v ^ (long long)s) - (long long)s);
+  const int lz = __clzll((long long)m);                                 // 2 .. 64
+  const unsigned long long n = (m << (lz & 63)) + 0x400;
+  unsigned long long bits = ((unsigned long long)(unsigned)(1045 - lz + e) << 52) + (n >> 11);   // (the leading bit adds one)
+  if (n < 0x400ull) bits = (unsigned long long)(unsigned)(1047 - lz + e) << 52;                  // a carry out of bit 63
+  if (m == 0 || e < -900) bits = 0;
+  return __longlong_as_double((long long)(bits | ((unsigned long long)(unsigned)s << 63 & 0x8000000000000000ull)));
+}
 // 2^e as a float for e <= 0, 0 below the normal range
 __device__ __forceinline__ float pow2_neg(int e) { return e < -126 ? 0.f : __int_as_float((e + 127) << 23); }
 
@@ -250,9 +267,14 @@ __global__ void __launch_bounds__(TTHREADS, 1)
       if (step % STEPS == 0 && step > 0) x[q].e += t < na ? ldea : ldeb;
       x[q].load(r_first + (long long)step * TBK < A.n);
     };
-    float hi[NQ], lo[NQ];
+    constexpr bool FP64 = ND >= 6;
+    float hi[NQ], lo[NQ];   // the sums of FP32 accuracy,
+    double sum[NQ];         // and of FP64 accuracy
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) hi[q] = lo[q] = 0.f;
+    for (int q = 0; q < NQ; ++q) {
+      hi[q] = lo[q] = 0.f;
+      sum[q] = 0.0;
+    }
     const int quarter = warp & 3, jq = (warp >> 2) * NQ;
     const int row = 32 * quarter + lane;
     const uint32_t tlane = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)jq;
@@ -262,7 +284,8 @@ __global__ void __launch_bounds__(TTHREADS, 1)
       const int ch = ch0 + chunk;
       // (a column of zeros in the chunk has no digits that mean anything)
       const int xa = i0 + row < i1 ? exponent_in(expA[(long long)ch * ldea + i0 + row]) : 0;
-      const float fa = xa ? pow2_neg(xa - ra[row]) : 0.f;
+      const int ea = xa ? xa - ra[row] : -4096;
+      const float fa = pow2_neg(ea);
 #pragma unroll
       for (int c0 = 0; c0 < NQ; c0 += 4) {
         float v[NW][4];
@@ -277,23 +300,34 @@ __global__ void __launch_bounds__(TTHREADS, 1)
         tmem_ld_wait();
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const float g = fa * pow2_neg(e[q]);
-          // three leading weights by error-free sums, the rest in one float
-          float s = hi[c0 + q], err = 0.f;
+          if constexpr (FP64) {
+            // in units of the sixth weight (rounded there); the weights are integers below 2^25
+            int i[NW];
 #pragma unroll
-          for (int w = 0; w < 3; ++w) {
-            const float t = v[w][q] * (g * (w == 0 ? 1.f : w == 1 ? 0x1p-8f : 0x1p-16f));
-            const float n = __fadd_rn(s, t), b = __fsub_rn(n, s);
-            err = __fadd_rn(err, __fadd_rn(__fsub_rn(s, __fsub_rn(n, b)), __fsub_rn(t, b)));
-            s = n;
+            for (int w = 0; w < NW; ++w) i[w] = __float2int_rn(v[w][q]);
+            const long long top = ((long long)i[0] << 40) + ((long long)i[1] << 32);
+            const long long mid = ((long long)i[2] << 24) + ((long long)i[3] << 16);
+            const int below = NW > 7 ? i[6] + ((i[NW - 1] + 128) >> 8) : i[6];
+            sum[c0 + q] += chunk_value(top + mid + ((long long)i[4] << 8) + i[5] + ((below + 128) >> 8), ea + e[q]);
+          } else {
+            const float g = fa * pow2_neg(e[q]);
+            // three leading weights by error-free sums, the rest in one float
+            float s = hi[c0 + q], err = 0.f;
+#pragma unroll
+            for (int w = 0; w < 3; ++w) {
+              const float t = v[w][q] * (g * (w == 0 ? 1.f : w == 1 ? 0x1p-8f : 0x1p-16f));
+              const float n = __fadd_rn(s, t), b = __fsub_rn(n, s);
+              err = __fadd_rn(err, __fadd_rn(__fsub_rn(s, __fsub_rn(n, b)), __fsub_rn(t, b)));
+              s = n;
+            }
+            float tail = v[NW - 1][q];
+#pragma unroll
+            for (int w = NW - 2; w >= 3; --w) tail = fmaf(tail, 0x1p-8f, v[w][q]);
+            const float l = __fadd_rn(lo[c0 + q], fmaf(tail, g * 0x1p-24f, err));
+            const float n = __fadd_rn(s, l);
+            lo[c0 + q] = __fsub_rn(l, __fsub_rn(n, s));
+            hi[c0 + q] = n;
           }
-          float tail = v[NW - 1][q];
-#pragma unroll
-          for (int w = NW - 2; w >= 3; --w) tail = fmaf(tail, 0x1p-8f, v[w][q]);
-          const float l = __fadd_rn(lo[c0 + q], fmaf(tail, g * 0x1p-24f, err));
-          const float n = __fadd_rn(s, l);
-          lo[c0 + q] = __fsub_rn(l, __fsub_rn(n, s));
-          hi[c0 + q] = n;
         }
       }
       tc_fence_before();
@@ -336,7 +370,7 @@ __global__ void __launch_bounds__(TTHREADS, 1)
         if (j >= j1) continue;
         const int e2 = rb[jq + q];
         const bool bad = lost || er >= 2047 || e2 >= 2047;  // infinities and NaN
-        out[j] = bad ? (double)NAN : scalbn((double)hi[q] + (double)lo[q], product_unit<ND>(er, e2));
+        out[j] = bad ? (double)NAN : scalbn(FP64 ? sum[q] : (double)hi[q] + (double)lo[q], product_unit<ND>(er, e2));
       }
     }
   }
