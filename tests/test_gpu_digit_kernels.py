@@ -92,3 +92,69 @@ def test_gram_non_finite_columns(digits, fp64):
     bad = np.zeros_like(G, dtype=bool)
     bad[136], bad[:, 15] = True, True
     assert np.array_equal(~np.isfinite(G), bad) and np.array_equal(G[~bad], ref[~bad])
+
+
+@pytest.mark.parametrize("beta,alpha,signed", [(0.0, 1.0, False), (1.0, -1.0, False), (-2.0, 1.0, True)])
+@pytest.mark.parametrize("P,Q,n", [(8, 4, 8192), (8, 8, 8193), (16, 9, 8319), (17, 16, 8320), (33, 20, 9000), (48, 24, 8193),
+                                   (73, 25, 8319), (74, 32, 8447), (80, 26, 8192), (80, 32, 20001)])
+def test_update_keeps_every_digit(P, Q, n, beta, alpha, signed):
+    """Integers of up to 37 bits beside a column of 2^45 that meets coefficients
+    of zero: rows are cut against the large column in units of 2^-9, the results
+    (below 2^53) come from the lower digits, and nothing is rounded.  Negative
+    values are one unit too low, in A (signed) 2^-9 at most, in C (alpha < 0)
+    2^-47."""
+    torch = need_torch_cuda()
+    rng = np.random.default_rng(P + 10 * Q + n)
+    top = (1 << 37) // (2 * P)
+    a = rng.integers(-top if signed else 0, top, size=(2 * P, n)).astype(np.float64)
+    big = int(rng.integers(0, 2 * P))
+    a[big] = 2.0 ** 45
+    a[big, ::3] = 0.0
+    C = rng.integers(0, 256, size=(2 * P, 2 * Q)).astype(np.float64)
+    C[big] = 0.0
+    C[:, 2 * Q - 1] = 0.0
+    y = rng.integers(-1000, 1001, size=(2 * Q, n)).astype(np.float64)
+    want = alpha * (C.T @ a) + beta * y    # (every product and sum an integer below 2^53)
+    tol = 0.0
+    if signed:
+        tol = np.where(C.any(0), 1.0 + 2.0 ** -9 * C.sum(0), 0.0)[:, None]
+    if alpha < 0:   # (2^37 bounds the sum of a row; and a rounding of as much again)
+        tol = 2.0 * 2.0 ** (37 - 47)
+    for tiny in (False, True):   # powers of two on rows (down to 1e-301) and on all of C
+        s, c = np.ones(n), 1.0
+        if tiny:
+            s[::7], s[1::7], c = 2.0 ** -1000, 2.0 ** -520, 2.0 ** 520
+        A = torch.from_numpy(_complex_columns(a * s)).cuda()
+        Ck, Y0, w = C * c, y * (s * c), want * (s * c)
+        Y = torch.from_numpy(_complex_columns(Y0)).cuda()
+        Y = torch.cat([Y, torch.full((1, n), 7.0, dtype=Y.dtype, device="cuda")])
+        Cd = torch.from_numpy(Ck).cuda()
+        e = _lib().bdg_kernel_update(A.data_ptr(), A.stride(0), P, Cd.data_ptr(), beta, alpha, Y.data_ptr(), n, Q, n,
+                                     torch.cuda.current_stream().cuda_stream)
+        assert e == 0
+        Yh = Y.cpu().numpy()
+        assert np.all(np.abs(_real_columns(Yh[:Q]) - w) <= tol * (s * c)), tiny
+        assert np.all(Yh[Q] == 7.0)
+
+
+def test_update_non_finite_rows_and_columns():
+    torch = need_torch_cuda()
+    g = torch.Generator(device="cuda").manual_seed(2)
+    A = torch.randn((24, 8200), dtype=torch.complex128, device="cuda", generator=g)
+    C = torch.randn((48, 50), dtype=torch.float64, device="cuda", generator=g)
+
+    def run():
+        Y = torch.zeros((25, 8200), dtype=torch.complex128, device="cuda")
+        assert _lib().bdg_kernel_update(A.data_ptr(), 8200, 24, C.data_ptr(), 0.0, 1.0, Y.data_ptr(), 8200, 25, 8200,
+                                        torch.cuda.current_stream().cuda_stream) == 0
+        return _real_columns(Y.cpu().numpy())
+
+    ref = run()
+    A[3, 17] = complex(float("nan"), 0.0)
+    A[23, 8199] = complex(0.0, float("inf"))
+    C[5, 31] = float("inf")
+    got = run()
+    bad = np.zeros_like(ref, dtype=bool)
+    bad[:, [17, 8199]] = True
+    bad[31] = True
+    assert np.array_equal(~np.isfinite(got), bad) and np.array_equal(got[~bad], ref[~bad])
