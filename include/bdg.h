@@ -139,11 +139,12 @@ bdg_status bdg_biortho(bdg_plan_t plan, int dtype, void* F, void* G, int ncol, c
  *   G       device, double[2 ncol_a][2 ncol_b] row-major:
  *           G[2i+s][2j+t] = sum_{r<n} part_s(A_i[r]) part_t(B_j[r]),
  *           part_0 the real and part_1 the imaginary part.
- *   engine  BDG_GRAM_SIMT: FP32 on the CUDA cores (C64), or FP64 accuracy,
- *           about 1e-15 of sum |a b| (C128): double-float on the CUDA cores,
- *           from 8192 rows on exact integer digits on the tensor cores, whose
- *           error is relative to each column's largest value among 256
- *           neighbouring rows; row chunks summed in FP64;
+ *   engine  BDG_GRAM_SIMT: FP32 (C64) or double-float with about 1e-15 of
+ *           sum |a b| (C128) on the CUDA cores, row chunks summed in FP64.
+ *           C128 blocks of 8192 rows and more take exact integer digits on
+ *           the tensor cores where those are at least as accurate for an
+ *           output (seven digits beside the columns' largest values among 256
+ *           rows: 2^-49 of sum |a b|), and double-float for the others;
  *           BDG_GRAM_TENSOR: every element split into three BF16 slices,
  *           the six leading slice products accumulated in FP32 by the
  *           tensor cores (tcgen05), row chunks summed in FP64: FP32 accuracy

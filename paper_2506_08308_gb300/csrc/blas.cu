@@ -106,12 +106,23 @@ __device__ __forceinline__ void df_fma(float& sh, float& sl, float ah, float al,
 // Partial Gram over one row chunk in double-float (layout as k_gram_partial),
 // output tile (16 MP) x (16 MQ) real columns so that narrow and 48-wide
 // blocks waste no arithmetic; with upper set (A and B tiled alike) only the
-// tiles on or above the diagonal are formed.
+// tiles on or above the diagonal are formed.  With a mask of the outputs (and
+// *any, whether one of them is wanted) only the tiles that hold a wanted one.
 template <int MP, int MQ>
 __global__ void __launch_bounds__(256) k_gram_partial_df(PairBlock<double> A, PairBlock<double> B,
-                                                         double* __restrict__ part, int upper, long long crows) {
+                                                         double* __restrict__ part, int upper, long long crows,
+                                                         const uint8_t* __restrict__ mask, const int* __restrict__ any) {
   constexpr int TP = 16 * MP, TQ = 16 * MQ;
   if (upper && blockIdx.y < blockIdx.x) return;
+  if (mask) {
+    if (!*any) return;
+    bool wanted = false;
+    for (int e = threadIdx.x; e < TP * TQ; e += 256) {
+      const int i = blockIdx.x * TP + e / TQ, j = blockIdx.y * TQ + e % TQ;
+      if (i < 2 * A.cols && j < 2 * B.cols && mask[(long long)i * 2 * B.cols + j]) wanted = true;
+    }
+    if (!__syncthreads_or(wanted)) return;
+  }
   __shared__ float sAh[GK][TP + 4], sAl[GK][TP + 4];
   __shared__ float sBh[GK][TQ + 4], sBl[GK][TQ + 4];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
@@ -194,14 +205,17 @@ inline int tile_mult(int n) {
 // read from their mirror (upper-triangle Grams)
 // in a fixed order: thread (x, y) of a 32 x 8 block sums chunks y, y + 8,
 // ... of one output (independent loads in flight), then the eight sums are
-// added in order of y
+// added in order of y; with a mask, of the wanted outputs only
 __global__ void __launch_bounds__(256) k_gram_reduce_upper(const double* __restrict__ part, int nchunks, int P2,
-                                                           int Q2, int tile, double* __restrict__ G) {
+                                                           int Q2, int tile, double* __restrict__ G,
+                                                           const uint8_t* __restrict__ mask, const int* __restrict__ any) {
+  if (mask && !*any) return;
   __shared__ double t[8][33];
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
   const int e = blockIdx.x * 32 + x, nout = P2 * Q2;
   double s = 0.0;
-  if (e < nout) {
+  const bool wanted = e < nout && (!mask || mask[e]);
+  if (wanted) {
     const int i = e / Q2, j = e - i * Q2;
     const int src = (i / tile > j / tile) ? j * Q2 + i : e;
 #pragma unroll 4
@@ -209,7 +223,7 @@ __global__ void __launch_bounds__(256) k_gram_reduce_upper(const double* __restr
   }
   t[y][x] = s;
   __syncthreads();
-  if (y == 0 && e < nout) {
+  if (y == 0 && wanted) {
     double g = t[0][x];
 #pragma unroll
     for (int q = 1; q < 8; ++q) g += t[q][x];
@@ -367,18 +381,85 @@ size_t gram_workspace_bytes(int P, int Q, long long n) {
   return sizeof(double) * (size_t)nchunks * (size_t)(2 * P) * (size_t)(2 * Q);
 }
 
-// Digits on the tensor cores or double-float on the FP32 pipes.  Measured at
-// n = 196608 (double-float -> digits): 72 x 72 pairs 2627 -> 523 us, 24 x 24
-// 736 -> 138, 3 x 24 373 -> 125; at n = 12288: 24 x 24 648 -> 44 us.  Below
-// 8192 rows (32 chunks of 256) there are too few row groups for the SMs and
-// the launches count; a single pair of columns has no tile to fill.
+// Digits on the tensor cores or double-float on the FP32 pipes.  Measured
+// (double-float -> seven digits / with the check) at n = 196608: 72 x 72 pairs 2627
+// -> 648 / 711 us, 24 x 24 534 -> 147 / 172, 3 x 24 281 -> 134 / 158; at n = 12288:
+// 24 x 24 49 -> 37 / 52, 48 x 48 107 -> 42 / 60.  Narrow blocks gain nothing (8 x 8
+// of 98304 rows 66 -> 63 / 77, 1 x 2 of 196608 82 -> 101 / 115) but are kept with the
+// others: digits hold columns of any size, double-float those within FP32's
+// range.  Below 8192 rows (32 chunks of 256) there are too few row groups for the
+// SMs and the launches count; a single pair of columns has no tile to fill.
 bool gram_digits_pays(int P, int Q, long long n) { return P * Q > 1 && n >= 8192; }
 
 cudaError_t gram_pairs_fp64(const PairBlock<double>& A, const PairBlock<double>& B, double* G_dev, void* ws,
-                            size_t ws_bytes, cudaStream_t s, bool upper, int digits) {
+                            size_t ws_bytes, cudaStream_t s, bool upper) {
   if (A.n == B.n && gram_digits_pays(A.cols, B.cols, A.n) && gram_digits_fits(A.cols, B.cols, A.n, ws_bytes))
-    return gram_pairs_digits<double>(A, B, digits, G_dev, ws, ws_bytes, s);
+    return gram_pairs_digits<double>(A, B, 7, G_dev, ws, ws_bytes, s);
   return gram_pairs<double>(A, B, G_dev, ws, ws_bytes, s, upper);
+}
+
+// Gram in double-float: all of it, or the outputs that mask and any ask for
+static cudaError_t gram_df(const PairBlock<double>& A, const PairBlock<double>& B, double* G_dev, void* ws, size_t ws_bytes,
+                           cudaStream_t s, bool upper, const uint8_t* mask, const int* any) {
+  const int P2 = 2 * A.cols, Q2 = 2 * B.cols;
+  int mp = tile_mult(P2), mq = tile_mult(Q2);
+  const bool up = upper && P2 == Q2;
+  if (up) mp = mq = std::max(mp, mq);
+  // narrow blocks have few output tiles: shorter row chunks (more CTAs, up
+  // to about four per SM) as far as the workspace holds their partial sums
+  const long long tiles = (long long)((P2 + 16 * mp - 1) / (16 * mp)) * ((Q2 + 16 * mq - 1) / (16 * mq));
+  long long crows = GROWS, nch = (A.n + GROWS - 1) / GROWS;
+  const long long want = (4 * 152 + tiles - 1) / tiles;
+  if (want > nch) {
+    const long long cap = (long long)(ws_bytes / (sizeof(double) * (size_t)P2 * Q2));
+    long long target = std::min(want, cap);
+    if (target > nch) {
+      crows = ((A.n + target - 1) / target + GK - 1) / GK * GK;
+      nch = (A.n + crows - 1) / crows;
+    }
+  }
+  if (nch > 65535) {   // gridDim.z
+    crows = ((A.n + 65534) / 65535 + GK - 1) / GK * GK;
+    nch = (A.n + crows - 1) / crows;
+  }
+  // The tile that the launch uses: smaller ones where the chunks leave SMs
+  // idle (a sum does not depend on the tile).  Clocks of a row of a CTA: 15
+  // instructions per multiply-add of 256 threads on four schedulers, the
+  // split of the operands on the FP64 pipe, and what does not shrink.  24 x 24
+  // pairs of 49152 rows (24 chunks) 658 -> 241 us; 72 x 72 pairs of 768 rows
+  // 329 -> 14 us, where the 64 x 64 tiles of one chunk ran on nine SMs.
+  {
+    long long best = -1;
+    int bp = mp, bq = mq;
+    for (int a = mp; a >= 1; --a)
+      for (int b = mq; b >= 1; --b) {
+        if (up && a != b) continue;
+        const long long tp = (P2 + 16 * a - 1) / (16 * a), tq = (Q2 + 16 * b - 1) / (16 * b);
+        const long long ctas = (up ? tp * (tp + 1) / 2 : tp * tq) * nch;
+        const long long cost = (ctas + 151) / 152 * (30 * a * b + 32 * (a + b) + 40);
+        if (best < 0 || cost < best) {
+          best = cost;
+          bp = a;
+          bq = b;
+        }
+      }
+    mp = bp;
+    mq = bq;
+  }
+  dim3 g8((P2 + 16 * mp - 1) / (16 * mp), (Q2 + 16 * mq - 1) / (16 * mq), (unsigned)nch);
+#define BDG_GDF(MP_, MQ_) \
+  if (mp == MP_ && mq == MQ_) k_gram_partial_df<MP_, MQ_><<<g8, 256, 0, s>>>(A, B, (double*)ws, up ? 1 : 0, crows, mask, any);
+  BDG_GDF(1, 1) BDG_GDF(1, 2) BDG_GDF(1, 3) BDG_GDF(1, 4)
+  BDG_GDF(2, 1) BDG_GDF(2, 2) BDG_GDF(2, 3) BDG_GDF(2, 4)
+  BDG_GDF(3, 1) BDG_GDF(3, 2) BDG_GDF(3, 3) BDG_GDF(3, 4)
+  BDG_GDF(4, 1) BDG_GDF(4, 2) BDG_GDF(4, 3) BDG_GDF(4, 4)
+#undef BDG_GDF
+  cudaError_t e8 = cudaGetLastError();
+  if (e8 != cudaSuccess) return e8;
+  const int nout8 = P2 * Q2;
+  k_gram_reduce_upper<<<(nout8 + 31) / 32, 256, 0, s>>>((const double*)ws, (int)nch, P2, Q2,
+                                                          up ? 16 * mp : (1 << 30), G_dev, mask, any);
+  return cudaGetLastError();
 }
 
 template <typename R>
@@ -392,62 +473,8 @@ cudaError_t gram_pairs(const PairBlock<R>& A, const PairBlock<R>& B, double* G_d
   if (ws_bytes < gram_workspace_bytes(A.cols, B.cols, A.n)) return cudaErrorInvalidValue;
   dim3 grid((P2 + GT - 1) / GT, (Q2 + GT - 1) / GT, (unsigned)nchunks);
   if (sizeof(R) == 8) {
-    const PairBlock<double>& A8 = *reinterpret_cast<const PairBlock<double>*>(&A);
-    const PairBlock<double>& B8 = *reinterpret_cast<const PairBlock<double>*>(&B);
-    int mp = tile_mult(P2), mq = tile_mult(Q2);
-    const bool up = upper && P2 == Q2;
-    if (up) mp = mq = std::max(mp, mq);
-    // narrow blocks have few output tiles: shorter row chunks (more CTAs, up
-    // to about four per SM) as far as the workspace holds their partial sums
-    const long long tiles = (long long)((P2 + 16 * mp - 1) / (16 * mp)) * ((Q2 + 16 * mq - 1) / (16 * mq));
-    long long crows = GROWS, nch = nchunks;
-    const long long want = (4 * 152 + tiles - 1) / tiles;
-    if (want > nch) {
-      const long long cap = (long long)(ws_bytes / (sizeof(double) * (size_t)P2 * Q2));
-      long long target = std::min(want, cap);
-      if (target > nch) {
-        crows = ((A.n + target - 1) / target + GK - 1) / GK * GK;
-        nch = (A.n + crows - 1) / crows;
-      }
-    }
-    // The tile that the launch uses: smaller ones where the chunks leave SMs
-    // idle (a sum does not depend on the tile).  Clocks of a row of a CTA: 15
-    // instructions per multiply-add of 256 threads on four schedulers, the
-    // split of the operands on the FP64 pipe, and what does not shrink.  24 x 24
-    // pairs of 49152 rows (24 chunks) 658 -> 241 us; 72 x 72 pairs of 768 rows
-    // 329 -> 14 us, where the 64 x 64 tiles of one chunk ran on nine SMs.
-    {
-      long long best = -1;
-      int bp = mp, bq = mq;
-      for (int a = mp; a >= 1; --a)
-        for (int b = mq; b >= 1; --b) {
-          if (up && a != b) continue;
-          const long long tp = (P2 + 16 * a - 1) / (16 * a), tq = (Q2 + 16 * b - 1) / (16 * b);
-          const long long ctas = (up ? tp * (tp + 1) / 2 : tp * tq) * nch;
-          const long long cost = (ctas + 151) / 152 * (30 * a * b + 32 * (a + b) + 40);
-          if (best < 0 || cost < best) {
-            best = cost;
-            bp = a;
-            bq = b;
-          }
-        }
-      mp = bp;
-      mq = bq;
-    }
-    dim3 g8((P2 + 16 * mp - 1) / (16 * mp), (Q2 + 16 * mq - 1) / (16 * mq), (unsigned)nch);
-#define BDG_GDF(MP_, MQ_) \
-  if (mp == MP_ && mq == MQ_) k_gram_partial_df<MP_, MQ_><<<g8, 256, 0, s>>>(A8, B8, (double*)ws, up ? 1 : 0, crows);
-    BDG_GDF(1, 1) BDG_GDF(1, 2) BDG_GDF(1, 3) BDG_GDF(1, 4)
-    BDG_GDF(2, 1) BDG_GDF(2, 2) BDG_GDF(2, 3) BDG_GDF(2, 4)
-    BDG_GDF(3, 1) BDG_GDF(3, 2) BDG_GDF(3, 3) BDG_GDF(3, 4)
-    BDG_GDF(4, 1) BDG_GDF(4, 2) BDG_GDF(4, 3) BDG_GDF(4, 4)
-#undef BDG_GDF
-    cudaError_t e8 = cudaGetLastError();
-    if (e8 != cudaSuccess) return e8;
-    const int nout8 = P2 * Q2;
-    k_gram_reduce_upper<<<(nout8 + 31) / 32, 256, 0, s>>>((const double*)ws, (int)nch, P2, Q2,
-                                                            up ? 16 * mp : (1 << 30), G_dev);
-    return cudaGetLastError();
+    return gram_df(*reinterpret_cast<const PairBlock<double>*>(&A), *reinterpret_cast<const PairBlock<double>*>(&B), G_dev, ws,
+                   ws_bytes, s, upper, nullptr, nullptr);
   }
   k_gram_partial<R><<<grid, 256, 0, s>>>(A, B, (double*)ws);
   cudaError_t e = cudaGetLastError();
@@ -455,6 +482,23 @@ cudaError_t gram_pairs(const PairBlock<R>& A, const PairBlock<R>& B, double* G_d
   const int nout = P2 * Q2;
   k_gram_reduce<<<(nout + 31) / 32, 256, 0, s>>>((const double*)ws, (int)nchunks, nout, G_dev);
   return cudaGetLastError();
+}
+
+// any and mask lie behind what the digits and the double-float sums need in turn
+static size_t checked_front_bytes(int P, int Q, long long n) {
+  return (std::max(gram_workspace_bytes(P, Q, n), gram_digits_checked_bytes(P, Q, n)) + 15) / 16 * 16;
+}
+size_t gram_checked_workspace_bytes(int P, int Q, long long n) {
+  return checked_front_bytes(P, Q, n) + 16 + (size_t)(2 * P) * (2 * Q);
+}
+cudaError_t gram_pairs_checked(const PairBlock<double>& A, const PairBlock<double>& B, double* G_dev, void* ws,
+                               size_t ws_bytes, cudaStream_t s) {
+  if (A.n != B.n || ws_bytes < gram_checked_workspace_bytes(A.cols, B.cols, A.n)) return cudaErrorInvalidValue;
+  const size_t front = checked_front_bytes(A.cols, B.cols, A.n);
+  int* any = (int*)((char*)ws + front);
+  uint8_t* mask = (uint8_t*)any + 16;
+  cudaError_t e = gram_digits_checked(A, B, G_dev, ws, front, mask, any, s);
+  return e != cudaSuccess ? e : gram_df(A, B, G_dev, ws, front, s, false, mask, any);
 }
 
 template <typename R>

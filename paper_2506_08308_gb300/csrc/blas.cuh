@@ -28,12 +28,18 @@ struct PairBlock {
 template <typename R>
 cudaError_t gram_pairs(const PairBlock<R>& A, const PairBlock<R>& B, double* G_dev, void* ws,
                        size_t ws_bytes, cudaStream_t s, bool upper = false);
-// FP64 Gram by digits where that pays (gram_digits_pays: long columns, more
-// than one pair), else by gram_pairs.  digits: 6, or 7 where 2^-48 of a
-// column's largest value in 256 rows is too much.
+// FP64 Gram by seven digits where that pays (gram_digits_pays: long columns, more
+// than one pair), else by gram_pairs.  The digits' error is relative to a column's
+// largest value in 256 rows: small beside |a| |b|.
 bool gram_digits_pays(int P, int Q, long long n);
 cudaError_t gram_pairs_fp64(const PairBlock<double>& A, const PairBlock<double>& B, double* G_dev, void* ws,
-                            size_t ws_bytes, cudaStream_t s, bool upper = false, int digits = 6);
+                            size_t ws_bytes, cudaStream_t s, bool upper = false);
+// The same with an error that is small beside sum |a b| for any columns: outputs
+// for which the digits may have lost more are formed again in double-float.  ws
+// must hold gram_checked_workspace_bytes.
+size_t gram_checked_workspace_bytes(int P, int Q, long long n);
+cudaError_t gram_pairs_checked(const PairBlock<double>& A, const PairBlock<double>& B, double* G_dev, void* ws,
+                               size_t ws_bytes, cudaStream_t s);
 size_t gram_workspace_bytes(int P, int Q, long long n);
 
 // The same Gram (full, no triangle) on the tensor cores with split-BF16
@@ -45,15 +51,19 @@ cudaError_t gram_pairs_tc(const PairBlock<R>& A, const PairBlock<R>& B, double* 
                           size_t ws_bytes, cudaStream_t s);
 
 // The same Gram (full, no triangle) from exact integer digits on the tensor
-// cores (gram_digits.cu): 6 or 7 of them for FP64 accuracy (FP64 blocks), 4
-// for FP32 accuracy.  ws as for
-// gram_pairs; fewer row groups run in parallel if it is short, and
-// gram_digits_fits says whether it holds one.
+// cores (gram_digits.cu): 7 of them for FP64 accuracy (FP64 blocks), 4 for FP32
+// accuracy.  ws as for gram_pairs; fewer row groups run in parallel if it is
+// short, and gram_digits_fits says whether it holds one.
 size_t gram_digits_workspace_bytes(int P, int Q, long long n);
 bool gram_digits_fits(int P, int Q, long long n, size_t ws_bytes);
 template <typename R>
 cudaError_t gram_pairs_digits(const PairBlock<R>& A, const PairBlock<R>& B, int digits, double* G_dev, void* ws,
                               size_t ws_bytes, cudaStream_t s);
+// Seven digits, and per output whether they may have lost more than 2^-49 of sum
+// |a b| (mask[e], and *any if one did); the part of gram_pairs_checked.
+size_t gram_digits_checked_bytes(int P, int Q, long long n);
+cudaError_t gram_digits_checked(const PairBlock<double>& A, const PairBlock<double>& B, double* G_dev, void* ws,
+                                size_t ws_bytes, uint8_t* mask, int* any, cudaStream_t s);
 
 // Y[:, q].t = beta * Y[:, q].t + alpha * sum_{p,s} A[:, p].s * C[(2p+s) * ldc + 2q+t]
 // C is FP64 on the device (row-major 2P x 2Q with leading dimension ldc);

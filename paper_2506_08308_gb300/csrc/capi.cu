@@ -569,11 +569,18 @@ bdg_status bdg_gram(int dtype, int engine, const void* A, long long lda, int nco
   if (engine == BDG_GRAM_TENSOR && !gram_tc_supported(ncol_a, ncol_b))
     return fail(nullptr, BDG_ERR_UNSUPPORTED, "tensor-core Gram needs 2 ncol_b <= 160");
   cudaStream_t s = (cudaStream_t)stream;
-  size_t ws_bytes = gram_workspace_bytes(ncol_a, ncol_b, n > 0 ? n : 1);
-  const bool digits = dtype == BDG_C128 && engine == BDG_GRAM_SIMT && gram_digits_pays(ncol_a, ncol_b, n);
-  if (digits) ws_bytes = std::max(ws_bytes, gram_digits_workspace_bytes(ncol_a, ncol_b, n));
+  const size_t plain_bytes = gram_workspace_bytes(ncol_a, ncol_b, n > 0 ? n : 1);
+  bool digits = dtype == BDG_C128 && engine == BDG_GRAM_SIMT && gram_digits_pays(ncol_a, ncol_b, n);
+  size_t ws_bytes = digits ? gram_checked_workspace_bytes(ncol_a, ncol_b, n) : plain_bytes;
   void* ws = nullptr;
-  if (cudaMallocAsync(&ws, ws_bytes, s) != cudaSuccess) {
+  cudaError_t em = cudaMallocAsync(&ws, ws_bytes, s);
+  if (em != cudaSuccess && digits) {   // the double-float Gram needs less
+    cudaGetLastError();
+    digits = false;
+    ws_bytes = plain_bytes;
+    em = cudaMallocAsync(&ws, ws_bytes, s);
+  }
+  if (em != cudaSuccess) {
     cudaGetLastError();
     return fail(nullptr, BDG_ERR_NOMEM, "Gram workspace allocation failed");
   }
@@ -581,7 +588,8 @@ bdg_status bdg_gram(int dtype, int engine, const void* A, long long lda, int nco
   if (dtype == BDG_C128) {
     PairBlock<double> a{(const double2*)A, lda, n, ncol_a}, b{(const double2*)B, ldb, n, ncol_b};
     e = engine == BDG_GRAM_TENSOR ? gram_pairs_tc<double>(a, b, G, ws, ws_bytes, s)
-                                  : gram_pairs_fp64(a, b, G, ws, ws_bytes, s);
+        : digits                  ? gram_pairs_checked(a, b, G, ws, ws_bytes, s)
+                                  : gram_pairs<double>(a, b, G, ws, ws_bytes, s, false);
   } else {
     PairBlock<float> a{(const float2*)A, lda, n, ncol_a}, b{(const float2*)B, ldb, n, ncol_b};
     e = engine == BDG_GRAM_TENSOR ? gram_pairs_tc<float>(a, b, G, ws, ws_bytes, s)

@@ -372,9 +372,9 @@ class Solver {
   // and the first pass of the two-pass Gram-Schmidt, whose second pass (FP64)
   // removes what the first leaves -- take four digits per element on the
   // tensor cores, the others seven where gram_digits_pays says so (else
-  // double-float; BDG_GRAM_TC=0: double-float and FP32 SIMT throughout).  Not
-  // six: the projected problems amplify what their Grams are off by, and on
-  // coarse grids the residuals of an FP64 solve level off near 1e-10.
+  // double-float; BDG_GRAM_TC=0: double-float and FP32 SIMT throughout).
+  // Columns are normalized, and what counts is an error that is small beside
+  // |a| |b| (gram_digits.cu: what it does to the residuals on coarse grids).
   bool tc_ = !getenv("BDG_GRAM_TC") || atoi(getenv("BDG_GRAM_TC")) != 0;
   static constexpr long long TC_MIN_ROWS = 2048;
   bdg_status gram(const PairBlock<R>& A, const PairBlock<R>& B, double* G, bool upper = false,
@@ -385,7 +385,7 @@ class Solver {
     }
     if constexpr (sizeof(R) == 8) {
       if (tc_) {
-        BDG_CUDA_TRY(plan_, gram_pairs_fp64(A, B, G, gws_, gws_bytes_, s_, upper, 7));
+        BDG_CUDA_TRY(plan_, gram_pairs_fp64(A, B, G, gws_, gws_bytes_, s_, upper));
         return BDG_OK;
       }
     }
