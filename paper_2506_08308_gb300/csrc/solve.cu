@@ -923,6 +923,7 @@ class Solver {
       cur_ = nxt;
       T* X = U_[cur_];
       T* HX = HU_[cur_];
+      if (sizeof(R) == 8 && it % 4 == 3 && (st = restore_biorthogonality(X, mmp, mm))) return st;
       if (exact_images_) {
         // images of the new Ritz block by the product itself: every residual
         // and every projected matrix then holds to the rounding of one product
@@ -1149,6 +1150,34 @@ class Solver {
     return BDG_OK;
   }
 
+  // The Ritz block X (mm real columns) is a combination of a basis with U^T V =
+  // I, by coefficients with P^T Q = I; nothing makes it bi-orthonormal again.
+  // Where one small eigenproblem comes out less accurate than the others, what
+  // F^T G = I + E is then off by stays, and every residual levels off near it
+  // (128^3, a start block with E = 2e-8 from the first iterations on: 5e-8).
+  // F <- F (I - E^T/2), G <- G (I - E/2) takes that to E^2; where E is at
+  // rounding level, as it is as a rule (3e-14 on 256^2), nothing changes.
+  // W is scratch.
+  bdg_status restore_biorthogonality(T* X, int mmp, int mm) {
+    HostMat S;
+    bdg_status st = gram_host(fpart(X, 0, mmp), mm, gpart(X, 0, mmp), mm, S);
+    if (st) return st;
+    HostMat a(2 * mmp, 2 * mmp), b(2 * mmp, 2 * mmp);
+    double worst = 0.0;
+    for (int i = 0; i < mm; ++i)
+      for (int j = 0; j < mm; ++j) {
+        const double e = S(i, j) - (i == j ? 1.0 : 0.0);
+        worst = std::max(worst, std::fabs(e));
+        a(j, i) = -0.5 * e;
+        b(i, j) = -0.5 * e;
+      }
+    if (log_) fprintf(stderr, "[bdg]   F^T G - I %.2e\n", worst);
+    if (!(worst > 1e-12 && worst < 0.1)) return BDG_OK;
+    BDG_CUDA_TRY(plan_, cudaMemcpyAsync(Wb_, X, sizeof(T) * (size_t)vlen_ * mmp, cudaMemcpyDeviceToDevice, s_));
+    if ((st = update(fpart(Wb_, 0, mmp), a, 1.0, fptr(X, 0), mmp))) return st;
+    return update(gpart(Wb_, 0, mmp), b, 1.0, gptr(X, 0), mmp);
+  }
+
   // Twice: W_f -= B_f (B_g^T W_f), W_g -= B_g (B_f^T W_g), images alike, for
   // the bi-orthonormal basis B = the first bp pairs of (Bk, HBk).
   bdg_status cgs2(const T* Bk, const T* HBk, int bp, T* W, T* HW, int wp) {
@@ -1160,7 +1189,7 @@ class Solver {
       const bool first_of_two = pass == 0 && cgs_passes_ >= 2;
       if ((st = gram(gpart(Bk, 0, bp), fpart(W, 0, wp), c1, false, sizeof(R) == 4 || first_of_two))) return st;
       if ((st = gram(fpart(Bk, 0, bp), gpart(W, 0, wp), c2, false, sizeof(R) == 4 || first_of_two))) return st;
-      // (the updates stay in double-float in both passes: rounding errors of
+      // (the updates have FP64 accuracy in both passes: rounding errors of
       // an FP32 update lie outside span(B), where the second pass cannot
       // remove them, and near convergence W is mostly along B, so they
       // swamp its remaining part -- tried, and the solves stalled)
