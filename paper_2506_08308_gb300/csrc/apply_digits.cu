@@ -16,8 +16,8 @@
 // and n + 128 meet a circulant and a skew-circulant of 128 points each, which
 // halves the products and costs integer additions only.
 //
-// What is lost: half a unit of 2^-55 of the line's largest value, of 2^-56 of
-// K[0], and the weights past the eighth -- below the rounding of the FFTs
+// What is lost: up to a unit of 2^-55 of the line's largest value, half one of 2^-55 of
+// K[0]'s power of two, and the weights past the eighth -- below the rounding of the FFTs
 // (2^-53 at each of its stages).  Against extended precision, relative to the
 // result, one axis, digits / FFT: noise 2.0e-16 / 2.9e-16 (N = 256), 2.1e-16 /
 // 2.7e-16 (128), noise under a Gaussian 2.3e-16 / 2.9e-16, smooth functions
@@ -27,7 +27,7 @@
 // of 64 real lines takes 14 us of MMAs, each bound by its 6 KB of operands at
 // 128 bytes per clock, and about 20 of integer work at 1.7 instructions a
 // clock, one after the other: tensor memory and shared memory hold one block
-// at a time), 310 us of coupling, 240 of which are the FP64 pipe's multiply-adds.
+// at a time), 310 us of coupling at 90 % of the FP64 pipe (FG, 24 vectors: 136 us).
 //
 // One CTA of sixteen warps per SM, 32 complex (64 real) lines a tile: the
 // warps load, fold and cut the digits of a block of 128 x 64 values (MMA B

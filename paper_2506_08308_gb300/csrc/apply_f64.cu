@@ -24,10 +24,10 @@ static cudaError_t axis_spread(const ApplyArgs<R>& g, int ax, cudaStream_t s) {
   BDG_DISPATCH_N(g.grid->n[ax], launch_axis_spread, g, ax, s)
 }
 
-// Axes of 128 and 256 points go to the tensor cores from 2048 lines on (64
+// Axes of 128 and 256 points go to the tensor cores above 2048 lines (64
 // tiles of 32; apply_digits.cu).  Measured per product, before -> digits:
-// 256^2 x 32 UV 3097 -> 1052 us, x 48 FG 4414 -> 1312, x 4 435 -> 162 (full
-// FFTs); x 2 (3072 lines) 226 -> 150, 128^2 x 4 114 -> 75 (spread FFTs);
+// 256^2 x 32 UV 3097 -> 1052 us, x 48 FG 4414 -> 1319, x 4 FG 435 -> 168 (full
+// FFTs); x 2 FG (3072 lines) 226 -> 95, 128^2 x 4 FG 114 -> 58 (spread FFTs);
 // 256^2 x 1 (1536 lines) 119, with digits 145: a tile takes 30 (N = 128) or 60
 // us whether or not every SM has one.
 constexpr long long DIGIT_LINES = 2048;

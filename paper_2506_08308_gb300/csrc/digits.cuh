@@ -7,9 +7,10 @@
 // most 15 bits, and the FP32 accumulator of tcgen05.mma (kind::f16) adds
 // such products without rounding as long as the sum stays below 2^24, that
 // is for (summed rows) x (digit pairs) <= 1024.  All digit pairs (i, j) of
-// equal i + j have equal weight and share one accumulator; pairs with i + j
-// >= ND lie below the last digit and are left out.  What is lost is the
-// quantization of the inputs, half a unit of the last digit.
+// equal i + j have equal weight and share one accumulator.  Pairs with i + j
+// >= ND lie below the last digit; with seven digits the first such weight is
+// kept as well, the others are left out.  What is lost is the cut of the inputs,
+// at most a unit of X (bits below are dropped, a negative value is one too low).
 #pragma once
 
 #include <cuda_fp16.h>

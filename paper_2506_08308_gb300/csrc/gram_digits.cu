@@ -14,7 +14,7 @@
 // added to an FP64 sum per output in registers.  (In one double-float sum, the
 // weights from the fourth on in one float, what 256 rows lost was 2^-47 of that
 // product, and of 288 FP64 solves of 64^2 problems 38 levelled off above their
-// tolerance of 1e-10; 18 with double-float Grams, one now.)  FP32 accuracy: the
+// tolerance of 1e-10; 18 with double-float Grams, one or two now.)  FP32 accuracy: the
 // leading three weights error-free into a double-float sum.  The CTA writes its
 // sums as FP64, and the CTAs' partial sums are added in FP64 in a fixed order.
 //

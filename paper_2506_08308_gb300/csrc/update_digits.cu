@@ -6,7 +6,7 @@
 // once per call by k_update_table); seven 8-bit digits each, the eight leading
 // digit weights (34 products) summed by tcgen05.mma over up to 160 real
 // columns, put together in 64-bit integers and scaled by the two exponents.
-// The error is that of rounding A's rows and C's columns to 2^-55 of their
+// The error is that of cutting A's rows and C's columns at 2^-55 of their
 // largest values, against 2^-48 per term in double-float (k_update_df, which
 // spends 15 FP32 instructions on a multiply-add and is bound by them).
 //
@@ -67,8 +67,10 @@ __global__ void __launch_bounds__(KMAX) k_update_table(const double* __restrict_
     o[d * N * KC] = __int2half_rn((int)(d == 0 ? u >> 48 : (u >> (8 * (ND - 1 - d))) & 0xFF) - 128);
 }
 
-// sums of the eight weights in units of the sixth (rounded there); all are
-// integers below 2^24 (160 terms x up to 7 pairs x 2^14)
+// sums of the eight weights in units of the sixth (rounded there).  All but the
+// seventh are integers below 2^24 whatever the digits (160 terms x up to 6 pairs x
+// 2^14); the seventh (7 pairs) may pass it from 147 real columns on and then be
+// off by a unit, 2^-62 of the two largest values' product.
 __device__ __forceinline__ long long weigh(const float (&c)[NW]) {
   int i[NW];
 #pragma unroll

@@ -2,8 +2,8 @@
 instances of the batched workload whose floor lies closest to the tolerance of
 1e-10 (14, 20, 56, 59), each with two ground states of different start
 spinors.  At most one of the eight may stall with some of its 16 pairs above
-the tolerance (one solve of 288 did when this was measured, 18 with Grams in
-double-float)."""
+the tolerance (one or two solves of 288 did when this was measured, 18 with
+Grams in double-float)."""
 import numpy as np
 import pytest
 
